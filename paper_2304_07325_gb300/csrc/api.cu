@@ -221,6 +221,7 @@ int rebuild(symba_pool *P) {
     memcpy(descs[d].ck, cur[d].ck, sizeof(descs[d].ck));
     memcpy(descs[d].ck2, cur[d].ck2, sizeof(descs[d].ck2));
     memcpy(descs[d].invdc, cur[d].invdc, sizeof(descs[d].invdc));
+    memcpy(descs[d].hk, cur[d].hk, sizeof(descs[d].hk));
   }
   CK(cudaMemcpyAsync(P->D.disks, descs.data(), sizeof(DiskDesc) * P->max_disks, cudaMemcpyHostToDevice, P->stream));
   invalidate_graph(P);
@@ -400,7 +401,6 @@ int pool_create(symba_pool **out, int max_disks, long long max_particles, long l
   A(&D.acc, 3 * n);
   A(&D.g_moff, gs); A(&D.g_mcnt, gs); A(&D.g_poff, gs); A(&D.g_pcnt, gs); A(&D.g_cur, gs);
   A(&D.gmem, n); A(&D.rec_items, gs); A(&D.rec_total, 1);
-  A(&D.lcache, (size_t)P->L.sms * SYM_REC_BPSM_MAX * 4 * SYM_PAIR_LC);   // any schedule
   A(&P->eacc, 4 * (SA_NDIG + 1)); A(&P->eout, 4);
   if (st != SYMBA_OK) { symba_pool_free(P); return st; }
   if (cudaMemsetAsync(D.blk_disk, 0xFF, sizeof(int) * (n / SYM_TILE + 1), P->stream) != cudaSuccess ||

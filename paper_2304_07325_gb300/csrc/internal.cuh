@@ -19,7 +19,6 @@
 
 #define SYM_TILE 32
 #define SYM_MAX_LEVELS 32
-#define SYM_PAIR_LC (16 * (SYM_MAX_LEVELS + 2))   // level-constant cache of one recursion warp
 #define SYM_REC_BPSM_MAX 2   // recursion CTAs per SM a schedule may ask for
 #define SA_NDIG 68  // 32-bit digits of the exact accumulator, digit k weighs 2^(32k - 1088)
 #ifndef SYM_MACRO_COLS
@@ -39,6 +38,7 @@ struct DiskDesc {
   double ck[SYM_MAX_LEVELS + 2];    // c_k = c_{k-1} / shell_ratio, c_0 = 1 (R_k = R_0 c_k)
   double ck2[SYM_MAX_LEVELS + 2];   // c_k^2
   double invdc[SYM_MAX_LEVELS + 2]; // 1 / (c_k - c_{k+1})
+  double hk[SYM_MAX_LEVELS + 2];    // sub-step of level k: hk[0] = dt, hk[k] = hk[k-1] / M
 };
 
 struct DiskStat {               // mutable per-system counters (device)
@@ -93,7 +93,6 @@ struct Dev {
   int *gmem;                    // members grouped by group (global particle indices)
   int *rec_items;               // recursion work list (global group slot)
   int *rec_total;               // number of items
-  double *lcache;               // [recursion warp][SYM_PAIR_LC] single-pair level constants
 };
 
 // --------------------------------------------------------------------------------------------

@@ -16,6 +16,12 @@ __global__ void k_setup_disk(Dev D, int d) {
   }
   for (int k = 0; k < SYM_MAX_LEVELS + 1; ++k) dd->invdc[k] = 1.0 / (dd->ck[k] - dd->ck[k + 1]);
   dd->invdc[SYM_MAX_LEVELS + 1] = 0.0;
+  // as the recursion forms it: for M a power of two the product with 1/M is exact
+  const double invM = 1.0 / (double)dd->M;
+  const bool pow2 = (dd->M & (dd->M - 1)) == 0;
+  dd->hk[0] = dd->dt;
+  dd->hk[1] = dd->dt / (double)dd->M;
+  for (int k = 2; k < SYM_MAX_LEVELS + 2; ++k) dd->hk[k] = pow2 ? dd->hk[k - 1] * invM : dd->hk[k - 1] / (double)dd->M;
   DiskStat *st = &D.stat[d];
   st->npairs = 0;
   st->ngroups = 0;
