@@ -222,6 +222,8 @@ int rebuild(symba_pool *P) {
     memcpy(descs[d].ck2, cur[d].ck2, sizeof(descs[d].ck2));
     memcpy(descs[d].invdc, cur[d].invdc, sizeof(descs[d].invdc));
     memcpy(descs[d].hk, cur[d].hk, sizeof(descs[d].hk));
+    descs[d].kex = cur[d].kex;
+    descs[d].keg = cur[d].keg;
   }
   CK(cudaMemcpyAsync(P->D.disks, descs.data(), sizeof(DiskDesc) * P->max_disks, cudaMemcpyHostToDevice, P->stream));
   invalidate_graph(P);
@@ -365,7 +367,7 @@ int pool_create(symba_pool **out, int max_disks, long long max_particles, long l
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, P->device) != cudaSuccess) { delete P; return SYMBA_E_CUDA; }
   P->L.sms = prop.multiProcessorCount;
-  P->L.trap_blocks = P->L.sms * trap_blocks_per_sm(precision);
+  P->L.trap_blocks = P->L.sms * trap_blocks_default(precision);
   P->L.rec_blocks = P->L.sms * recursion_blocks_per_sm();
   if (!order_groups_init()) {
     if (P->own_stream) cudaStreamDestroy(P->stream);

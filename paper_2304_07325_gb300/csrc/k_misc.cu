@@ -1,5 +1,6 @@
 // O(N) kernels of the step: set-up, sun drift, partial-sum reduction with the kick, Kepler drift,
 // exact total momentum, state transfer and the energy diagnostic.
+#include "df32.cuh"
 #include "internal.cuh"
 
 // --------------------------------------------------------------------------------------------
@@ -73,18 +74,26 @@ void launch_discard(const Dev &D, long long npart, cudaStream_t s) {
 // and Hill radii rH_i = a_i (m_i / 3 m0)^{1/3} from the osculating heliocentric orbit
 // (vis-viva 1/a = 2/r - v^2/mu, mu = G (m0 + m_i); r if unbound; correctly rounded cube root).
 // --------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const double *vh,
+__global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const double *xh, const double *vh,
                                                    const double *m, double *q_out) {
   __shared__ unsigned long long acc[4][SA_NDIG + 1];
+  __shared__ int top[2];                  // high words of the largest |x| component and |G m|
+  if (threadIdx.x < 2) top[threadIdx.x] = 0;
   for (int k = threadIdx.x; k < 4 * (SA_NDIG + 1); k += blockDim.x) (&acc[0][0])[k] = 0ull;
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const double mi = m[i];
     sa_add(acc[3], mi);
-    for (int c = 0; c < 3; ++c) sa_add(acc[c], __dmul_rn(mi, vh[3 * i + c]));
+    for (int c = 0; c < 3; ++c) {
+      sa_add(acc[c], __dmul_rn(mi, vh[3 * i + c]));
+      atomicMax(&top[0], __double2hiint(xh[3 * i + c]) & 0x7FFFFFFF);
+    }
+    atomicMax(&top[1], __double2hiint(__dmul_rn(D.disks[d].G, mi)) & 0x7FFFFFFF);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    D.disks[d].kex = (top[0] >> 20) - 1023;
+    D.disks[d].keg = top[1] ? (top[1] >> 20) - 1023 : 0;
     const DiskDesc dd = D.disks[d];
     const double Mt = sa_round(acc[3]);
     const double denom = __dadd_rn(dd.m0, Mt);
@@ -139,7 +148,7 @@ void launch_init_state(const Dev &D, int d, int n, const double *xh, const doubl
                        cudaStream_t s) {
   // q (3 doubles) lives in the momentum slot of the system until the first momentum pass
   double *q = D.P + 3 * d;
-  k_init_sums<<<1, 256, 0, s>>>(D, d, n, vh, m, q);
+  k_init_sums<<<1, 256, 0, s>>>(D, d, n, xh, vh, m, q);
   k_init_state<<<64, 256, 0, s>>>(D, d, n, xh, vh, m, rad, rh, compute_rh, q);
 }
 
@@ -274,31 +283,36 @@ __global__ void k_reduce(Dev D, long long npart) {
     if (B >= dd.nbm) continue;                  // a block of field particles: kicked by k_field_*
     const int C = SYM_MACRO_COLS, ng = (dd.nbm + C - 1) / C, qB = B >> 2, gB = B / C;
     const int rslot = (B & 3) * 96 + lane, cslot = 384 + (B % C) * 96 + lane;
-    // the partials of p in a fixed order (its rows, then its columns); two interleaved sums
-    // (even and odd terms) keep two loads in flight, combined at the end
+    // the partials of p, double-float in the kick's units, in a fixed order (its rows, then its
+    // columns); two interleaved sums (even and odd terms) keep two loads in flight
     const int g0 = (4 / C) * qB, nrow = ng - g0;
     const int nterm = nrow + qB + 1;
-    auto ptr = [&](int t) -> const double * {
-      if (t < nrow) return D.part + (size_t)macro_index(dd, ng, qB, g0 + t) * SYM_MACRO_PART + rslot;
+    const float2 *part = reinterpret_cast<const float2 *>(D.part);
+    auto ptr = [&](int t) -> const float2 * {
+      if (t < nrow) return part + (size_t)macro_index(dd, ng, qB, g0 + t) * SYM_MACRO_PART + rslot;
       const int q = t - nrow;
-      return D.part + (size_t)macro_index(dd, ng, q, gB) * SYM_MACRO_PART + cslot;
+      return part + (size_t)macro_index(dd, ng, q, gB) * SYM_MACRO_PART + cslot;
     };
-    double ax0 = 0.0, ay0 = 0.0, az0 = 0.0, ax1 = 0.0, ay1 = 0.0, az1 = 0.0;
+    df s0[3], s1[3];
+    for (int k = 0; k < 3; ++k) s0[k] = s1[k] = mk(0.0f, 0.0f);
     int t = 0;
     for (; t + 1 < nterm; t += 2) {
-      const double *p0 = ptr(t), *p1 = ptr(t + 1);
-      ax0 += p0[0]; ay0 += p0[32]; az0 += p0[64];
-      ax1 += p1[0]; ay1 += p1[32]; az1 += p1[64];
+      const float2 *p0 = ptr(t), *p1 = ptr(t + 1);
+      for (int k = 0; k < 3; ++k) {
+        const float2 u = p0[32 * k], w = p1[32 * k];
+        s0[k] = add(s0[k], mk(u.x, u.y));
+        s1[k] = add(s1[k], mk(w.x, w.y));
+      }
     }
     if (t < nterm) {
-      const double *p0 = ptr(t);
-      ax0 += p0[0]; ay0 += p0[32]; az0 += p0[64];
+      const float2 *p0 = ptr(t);
+      for (int k = 0; k < 3; ++k) s0[k] = add(s0[k], mk(p0[32 * k].x, p0[32 * k].y));
     }
-    const double ax = ax0 + ax1, ay = ay0 + ay1, az = az0 + az1;
     const double h = 0.5 * dd.dt;
-    D.vx[p] = __dadd_rn(D.vx[p], __dmul_rn(h, ax));
-    D.vy[p] = __dadd_rn(D.vy[p], __dmul_rn(h, ay));
-    D.vz[p] = __dadd_rn(D.vz[p], __dmul_rn(h, az));
+    const int sc = dd.keg - 2 * dd.kex;
+    D.vx[p] = __dadd_rn(D.vx[p], __dmul_rn(h, kick_value(add(s0[0], s1[0]), sc)));
+    D.vy[p] = __dadd_rn(D.vy[p], __dmul_rn(h, kick_value(add(s0[1], s1[1]), sc)));
+    D.vz[p] = __dadd_rn(D.vz[p], __dmul_rn(h, kick_value(add(s0[2], s1[2]), sc)));
   }
 }
 

@@ -6,35 +6,40 @@
 // trapezoid becomes a rectangle of off-diagonal tiles plus the diagonal tiles of the triangle.
 // Tiles are grouped into macro-tiles of 4 row blocks (a 128-body quad q) by SYM_MACRO_COLS column
 // blocks (column group p, p >= 4q / SYM_MACRO_COLS), all macro-tiles of all systems in one flat
-// list that persistent CTAs of four warps consume from a counter (the fold of the triangle into a
-// rectangle, done by a work queue instead of index arithmetic).
+// list that persistent CTAs consume from a counter (the fold of the triangle into a rectangle, done
+// by a work queue instead of index arithmetic).
 //
-// One CTA per macro-tile, one warp per row block: warp w keeps row particle (4q + w)*32 + l in
-// lane l and sweeps the macro's column blocks in turn; in each tile lane l meets column
-// (l + s) mod 32 at step s (32 steps; 16 on a diagonal tile, where each unordered pair is met
-// once).  In the FP64 path the tile's column bodies are staged in the warp's shared memory and
-// only their accumulators rotate through the lanes by warp shuffle; the mixed path rotates the
-// bodies with them.  After the sweep every column accumulator is back in its home lane.  The row accumulators run on across the
-// macro-tile's tiles and are written once per macro-tile; the four warps' column accumulators of
-// each column block are added in shared memory in warp order and written once.  Both kinds of partials are
-// summed later in a fixed order: the result does not depend on scheduling, on how many
-// macro-tiles a CTA takes per grab, or on which other systems share the launch.
+// One CTA per macro-tile: a warp keeps row particle I*32 + l in lane l and sweeps the macro's column
+// blocks in turn; in each tile lane l meets column (l + s) mod 32 at step s (32 steps; 16 on a
+// diagonal tile, where each unordered pair is met once).  The column sums rotate through the lanes
+// by warp shuffle (the mixed path rotates the bodies with them).  The row accumulators run on across
+// the macro-tile's tiles; row and column sums of the CTA's warps are added in shared memory in warp
+// order and written once per macro-tile.  Both kinds of partials are summed later in a fixed order:
+// the result does not depend on scheduling, on how many macro-tiles a CTA takes per grab, or on
+// which other systems share the launch.
 //
-// FP64 path: 16 FP64-pipe instructions per pair (3 differences, 3 for r^2, 2 for r^-3 -- its seed,
-// Newton step and powers run on the integer pipe -- 2 mass scalings, 6 FMAs into the two
-// accumulators).
+// FP64 systems form the pair force in double-float (df32.cuh) on the FP32 pipe, which GB300 runs at
+// 62x the FP64 rate.  Separations come from coordinates cut on grids common to a macro-tile, exact
+// to 2^-61 of its extent; r^-3, the products and the sums carry 46 to 48 bits.  A kick is a small part
+// of v (a body of 1e-3 m0 at 1 AU and tau = 0.5 yr: 1/300), so its 2^-46 lies below the rounding
+// of v += (tau/2) a that follows; against an 80-bit kick the new v is as close as the FP64 pairs' was.
+//   10,000 bodies, per kick: 1.48 ms with 16.5 FP64 instructions per pair (FP64 pipe 90 % busy) ->
+//   0.55-0.58 ms with ~260 warp instructions per 32 pairs (61 % of the issue slots; four barriers per
+//   macro-tile take most of the rest).  1,000 bodies 0.160 -> 0.021 ms, 100 bodies 0.065 -> 0.017 ms
+//   (see k_trap_df and launch_trap for the small systems).
 //
 // Kick 1 also runs the close-encounter check (Sec. 2) of every pair: a conservative FP32
 // prefilter (|d| - tau |dv| against R_0 with rounding margins) and, for the rare pairs that pass,
 // the exact FP64 predicate, identical operation for operation to the definition; flagged pairs
 // are appended to the system's pair list and weighted by g_0(r).  Kick 2 weights the same
 // flagged pairs, found through the group each particle belongs to.
+#include "df32.cuh"
 #include "internal.cuh"
 
 #define FULL 0xffffffffu
 
 struct TileCtx {
-  int off, n, nm, pair_base, pair_cap, l;
+  int off, n, nm, pair_base, pair_cap, l, kex, keg;
   double dt, lam, c0, c1;
 };
 
@@ -42,6 +47,7 @@ __device__ __forceinline__ TileCtx load_ctx(const DiskDesc *dp) {
   TileCtx c;
   c.off = dp->off; c.n = dp->n; c.nm = dp->nm;
   c.pair_base = dp->pair_base; c.pair_cap = dp->pair_cap; c.l = dp->l;
+  c.kex = dp->kex; c.keg = dp->keg;
   c.dt = dp->dt; c.lam = dp->hill_scale; c.c0 = dp->ck[0]; c.c1 = dp->ck[1];
   return c;
 }
@@ -67,25 +73,70 @@ __device__ __forceinline__ bool group_has_pair(const Dev &D, int g, int lo, int 
 __device__ __forceinline__ size_t part_row(int m, int w) { return (size_t)m * SYM_MACRO_PART + w * 96; }
 __device__ __forceinline__ size_t part_col(int m, int k) { return (size_t)m * SYM_MACRO_PART + 384 + k * 96; }
 #define MC SYM_MACRO_COLS
+__device__ __forceinline__ df ld2(const float2 &v) { return mk(v.x, v.y); }
+
+// ---- FP64 systems: the pair arithmetic in double-float --------------------------------------------
+// A coordinate as three FP32 numbers on grids common to a tile: x = a + b + c with a a multiple of
+// 2^(E - 21), b in [0, 2^(E - 21)) of 2^(E - 41), c in [0, 2^(E - 41)) of 2^(E - 61), for |x| < 2^(E + 1).
+// Differences of a, of b and of c are exact, so a separation keeps every digit that matters down to
+// 2^-61 of the tile's extent in that component (FP64 positions of that size are multiples of 2^-52).
+// Values are scaled by 2^-kex.
+__device__ __forceinline__ void on_grid(double x, int E, int kex, float &a, float &b, float &c) {
+  const long long bits = __double_as_longlong(x);
+  const int e = (int)((bits >> 52) & 0x7FF) - 1023;
+  const unsigned long long man = (bits & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+  const int sh = 9 - (E - e);
+  unsigned long long u = sh >= 0 ? man << (sh & 63) : man >> min(-sh, 63);
+  if (e == -1023) u = 0ull;
+  const long long X = bits < 0 ? -(long long)u : (long long)u;       // x 2^(61 - E)
+  const float sa = __int_as_float((E - kex - 21 + 127) << 23);
+  a = __int2float_rn((int)(X >> 40)) * sa;
+  b = __int2float_rn((int)((X >> 20) & 0xFFFFF)) * (sa * 9.5367432e-7f);                   // 2^-20
+  c = __int2float_rn((int)(X & 0xFFFFF)) * (sa * 9.0949470e-13f);                          // 2^-40
+}
+// exponent of the grid of a component: that of its largest |x| (biased as in hi, the largest high
+// word), not below 2^-60 of the system's scale
+__device__ __forceinline__ int grid_exp(int hi, int kex) { return max((hi >> 20) - 1023, kex - 60); }
+__device__ __forceinline__ df separation(float aj, float bj, float cj, float ai, float bi, float ci) {
+  const df t = fast_two_sum(__fsub_rn(aj, ai), __fsub_rn(bj, bi));   // |da| >= |db| or da = 0
+  return fast_two_sum(t.h, __fadd_rn(t.l, __fsub_rn(cj, ci)));
+}
+// sum += t, the sum's low part collecting errors (48 bits of the sum)
+__device__ __forceinline__ void accumulate(df &sum, df t) {
+  const df s = two_sum(sum.h, t.h);
+  sum.h = s.h;
+  sum.l = __fadd_rn(sum.l, __fadd_rn(s.l, t.l));
+}
 
 // the row side of one warp: row particle I*32 + lane, its data and its accumulators
-struct RowF64 {
+struct RowDF {
   int pi;
   bool live, row;          // a live body; live and massive (a row of the trapezoid)
-  double x, y, z, ngm;     // position and -G m of the row body
+  float x[3][3];           // a, b, c of each component
+  df ngm;                  // -G m, scaled
   float xf, yf, zf, vxf, vyf, vzf, lam, sig;   // kick 1: FP32 prefilter copies
   int gid;                 // kick 2: encounter group
-  double ax, ay, az;       // carried across the macro-tile's column blocks
+  df acc[3];               // carried across the macro-tile's column blocks
+};
+
+// a column body in shared memory: {x: a b c, y: a} {y: b c, z: a b} {z: c, G m: h l, group}
+struct ColDF {
+  float4 q[3];
 };
 
 template <int MODE>
-__device__ __forceinline__ void row_load_fp64(const Dev &D, const TileCtx &c, int I, int lane, RowF64 &r) {
+__device__ __forceinline__ void row_load_df(const Dev &D, const TileCtx &c, const int *E, int I, int lane, RowDF &r) {
   r.pi = I * 32 + lane;
   const int li = r.pi - c.off;
   r.live = li < c.n && D.alive[r.pi];
   r.row = r.live && li < c.nm;
-  r.x = D.x[r.pi]; r.y = D.y[r.pi]; r.z = D.z[r.pi];
-  r.ngm = __longlong_as_double(__double_as_longlong(D.gm[r.pi]) ^ (long long)0x8000000000000000ull);
+  const double p[3] = {D.x[r.pi], D.y[r.pi], D.z[r.pi]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    on_grid(r.live ? p[k] : 0.0, E[k], c.kex, r.x[k][0], r.x[k][1], r.x[k][2]);
+    r.acc[k] = mk(0.0f, 0.0f);
+  }
+  r.ngm = neg(split(scale2(D.gm[r.pi], -c.keg)));
   r.xf = r.yf = r.zf = r.vxf = r.vyf = r.vzf = r.lam = r.sig = 0.f;
   r.gid = -1;
   if (MODE == 1) {
@@ -95,86 +146,49 @@ __device__ __forceinline__ void row_load_fp64(const Dev &D, const TileCtx &c, in
   } else {
     r.gid = D.gid[r.pi];
   }
-  r.ax = r.ay = r.az = 0.0;
 }
 
-// One warp's copy of a tile's 32 column bodies in shared memory.
-struct JStage {
-  double2 xy[32], zg[32];   // x, y | z, G m
-  float4 fa[32], fb[32];    // kick 1: the FP32 copies xf, yf, zf, vxf | vyf, vzf, lambda, sigma
-  int gid[32];              // kick 2: encounter group
-};
+// s w for the level-0 weight of a flagged pair (zero also where r^-3 left the FP32 range)
+__device__ __forceinline__ df weighted(df s, double w) { return w == 0.0 ? mk(0.0f, 0.0f) : mul(s, split(w)); }
 
-// One 32 x 32 tile (rows of block I, columns of block J >= I): both reactions of every pair;
-// the row side goes into r.ax.., the column side comes back in cx, cy, cz (zero on a diagonal
-// tile, whose column side is folded into its rows).  The column bodies are staged in js once;
-// at step s lane l takes column (l + s + o) mod 32 (o = 1 on a diagonal tile), whose column-side
-// sums travel with it from lane to lane.
+// Steps [t0, t1) of one 32 x 32 tile (rows of block I, columns of block J >= I, 32 steps; 16 on the
+// diagonal): at step t lane l meets column (l + t + o) mod 32 (o = 1 on the diagonal), whose
+// column-side sums travel with it from lane to lane.  The row side goes into r.acc, the column side
+// into out[component][column].
 template <int MODE>
-__device__ __forceinline__ void tile_sweep_fp64(const Dev &D, const TileCtx &c, int sys, RowF64 &r,
-                                                int I, int J, int lane, JStage *js, double &cx,
-                                                double &cy, double &cz) {
+__device__ __forceinline__ void tile_steps_df(const Dev &D, const TileCtx &c, int sys, RowDF &r, int I, int J, int lane,
+                                              int t0, int t1, const ColDF *col, const float4 (*cf)[2],
+                                              unsigned mlive, unsigned mmass, float2 (*out)[32]) {
   const bool diag = I == J;
-  {
-    const int j0 = J * 32 + lane;
-    __syncwarp();                         // the last tile's reads of js are done
-    js->xy[lane] = make_double2(D.x[j0], D.y[j0]);
-    js->zg[lane] = make_double2(D.z[j0], D.gm[j0]);
-    if (MODE == 1) {
-      js->fa[lane] = make_float4(D.xf[j0], D.yf[j0], D.zf[j0], D.vxf[j0]);
-      js->fb[lane] = make_float4(D.vyf[j0], D.vzf[j0], D.lamf[j0], D.sigf[j0]);
-    } else {
-      js->gid[lane] = D.gid[j0];
-    }
-  }
-  const int lj0 = J * 32 + lane - c.off;
-  const bool live_j0 = lj0 < c.n && D.alive[J * 32 + lane];
-  const unsigned mlive = __ballot_sync(FULL, live_j0), mmass = __ballot_sync(FULL, live_j0 && lj0 < c.nm);
-  __syncwarp();
-  double axj = 0.0, ayj = 0.0, azj = 0.0;
+  const int o = diag ? 1 : 0;
   const float tauf = __double2float_ru(c.dt);
-
-  auto rotate = [&]() {
-    const int src = (lane + 1) & 31;
-    axj = __shfl_sync(FULL, axj, src); ayj = __shfl_sync(FULL, ayj, src);
-    azj = __shfl_sync(FULL, azj, src);
-  };
-
-  const int nsteps = diag ? 16 : 32, o = diag ? 1 : 0;
+  df ca[3] = {mk(0.0f, 0.0f), mk(0.0f, 0.0f), mk(0.0f, 0.0f)};
 #pragma unroll 1
-  for (int s = 0; s < nsteps; ++s) {
-    const int cj = (lane + s + o) & 31;
+  for (int t = t0; t < t1; ++t) {
+    const int cj = (lane + t + o) & 31;
     const int jid = J * 32 + cj;
-    const int jflags = (int)((mlive >> cj) & 1u) | (int)(((mmass >> cj) & 1u) << 1);
-    const double2 q0 = js->xy[cj], q1 = js->zg[cj];
-    const double xj = q0.x, yj = q0.y, zj = q1.x, gmj = q1.y;
-    float xfj = 0.f, yfj = 0.f, zfj = 0.f, vxfj = 0.f, vyfj = 0.f, vzfj = 0.f, lamj = 0.f, sigj = 0.f;
-    int gidj = -1;
-    if (MODE == 1) {
-      const float4 fa = js->fa[cj], fb = js->fb[cj];
-      xfj = fa.x; yfj = fa.y; zfj = fa.z; vxfj = fa.w;
-      vyfj = fb.x; vzfj = fb.y; lamj = fb.z; sigj = fb.w;
-    } else {
-      gidj = js->gid[cj];
-    }
+    const bool jl = (mlive >> cj) & 1u, jm = (mmass >> cj) & 1u;
+    const float4 q0 = col[cj].q[0], q1 = col[cj].q[1], q2 = col[cj].q[2];
     bool valid;
     if (!diag) {
-      valid = r.row && (jflags & 1);
+      valid = r.row && jl;
     } else {
-      valid = (jid > r.pi) ? (r.row && (jflags & 1)) : (r.live && (jflags & 2));
-      if (s == 15 && lane >= 16) valid = false;  // pair {l, l+16} belongs to lane l < 16
+      valid = (jid > r.pi) ? (r.row && jl) : (r.live && jm);
+      if (t == 15 && lane >= 16) valid = false;  // pair {l, l+16} belongs to lane l < 16
     }
-    const double dx = xj - r.x, dy = yj - r.y, dz = zj - r.z;
-    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const double r3 = rinv3(r2);
-    double sj = gmj * r3;
-    double si = r.ngm * r3;             // the column side's -G m_i / r^3
+    const df d[3] = {separation(q0.x, q0.y, q0.z, r.x[0][0], r.x[0][1], r.x[0][2]),
+                     separation(q0.w, q1.x, q1.y, r.x[1][0], r.x[1][1], r.x[1][2]),
+                     separation(q1.z, q1.w, q2.x, r.x[2][0], r.x[2][1], r.x[2][2])};
+    const df r3 = inverse_cube(root(norm2(d)));
+    df sj = mul(mk(q2.y, q2.z), r3);
+    df si = mul(r.ngm, r3);             // the column side's -G m_i / r^3
     if (MODE == 1) {
-      const float dxf = xfj - r.xf, dyf = yfj - r.yf, dzf = zfj - r.zf;
+      const float4 fa = cf[cj][0], fb = cf[cj][1];
+      const float dxf = fa.x - r.xf, dyf = fa.y - r.yf, dzf = fa.z - r.zf;
       const float r2f = fmaf(dzf, dzf, fmaf(dyf, dyf, dxf * dxf));
-      const float dvxf = vxfj - r.vxf, dvyf = vyfj - r.vyf, dvzf = vzfj - r.vzf;
+      const float dvxf = fa.w - r.vxf, dvyf = fb.x - r.vyf, dvzf = fb.y - r.vzf;
       const float vmag = sqrtf(fmaf(dvzf, dvzf, fmaf(dvyf, dvyf, dvxf * dvxf)));
-      const float Bf = fmaf(tauf, vmag, r.lam + lamj) * 1.0000039f + 1.9073486e-6f * (r.sig + sigj);
+      const float Bf = fmaf(tauf, vmag, r.lam + fb.z) * 1.0000039f + 1.9073486e-6f * (r.sig + fb.w);
       const bool cand = valid && !(r2f > Bf * Bf);
       if (__any_sync(FULL, cand)) {
         if (cand) {
@@ -192,36 +206,42 @@ __device__ __forceinline__ void tile_sweep_fp64(const Dev &D, const TileCtx &c, 
             }
             const double er2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
             const double w = g0_weight(c, R0, __dsqrt_rn(er2));
-            sj *= w;
-            si *= w;
+            sj = weighted(sj, w);
+            si = weighted(si, w);
           }
         }
+        __syncwarp();
       }
     } else {
-      if (r.gid >= 0 && r.gid == gidj && valid) {
+      if (r.gid >= 0 && r.gid == __float_as_int(q2.w) && valid) {
         const int lo = min(r.pi, jid), hi = max(r.pi, jid);
         if (group_has_pair(D, r.gid, lo, hi)) {
           const double R0 = __dmul_rn(c.lam, __dadd_rn(D.rh[lo], D.rh[hi]));
-          const double w = g0_weight(c, R0, sqrt(r2));
-          sj *= w;
-          si *= w;
+          const double ex = D.x[hi] - D.x[lo], ey = D.y[hi] - D.y[lo], ez = D.z[hi] - D.z[lo];
+          const double w = g0_weight(c, R0, sqrt(fma(ez, ez, fma(ey, ey, ex * ex))));
+          sj = weighted(sj, w);
+          si = weighted(si, w);
         }
       }
     }
-    sj = keep_or_zero(sj, valid);
-    si = keep_or_zero(si, valid);
-    r.ax = fma(sj, dx, r.ax); r.ay = fma(sj, dy, r.ay); r.az = fma(sj, dz, r.az);
-    axj = fma(si, dx, axj); ayj = fma(si, dy, ayj); azj = fma(si, dz, azj);
-    if (!diag || s + 1 < nsteps) rotate();
+    sj.h = valid ? sj.h : 0.0f; sj.l = valid ? sj.l : 0.0f;
+    si.h = valid ? si.h : 0.0f; si.l = valid ? si.l : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      accumulate(r.acc[k], mul(sj, d[k]));
+      accumulate(ca[k], mul(si, d[k]));
+    }
+    if (t + 1 < t1) {
+      const int src = (lane + 1) & 31;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) ca[k] = mk(__shfl_sync(FULL, ca[k].h, src), __shfl_sync(FULL, ca[k].l, src));
+    }
   }
-  if (diag) {
-    const int src = (lane + 16) & 31;
-    r.ax += __shfl_sync(FULL, axj, src);
-    r.ay += __shfl_sync(FULL, ayj, src);
-    r.az += __shfl_sync(FULL, azj, src);
-    cx = 0.0; cy = 0.0; cz = 0.0;
-  } else {
-    cx = axj; cy = ayj; cz = azj;
+  const int last = (lane + t1 - 1 + o) & 31;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const df q = t1 > t0 ? renorm(ca[k]) : ca[k];
+    out[k][last] = make_float2(q.h, q.l);
   }
 }
 
@@ -381,21 +401,30 @@ __device__ __forceinline__ void tile_sweep_mixed(const Dev &D, const TileCtx &c,
   }
 }
 
-// One CTA (four warps) per macro-tile.  The macro-tile list entry is {system, first row block,
-// first column block, end of the system's massive blocks}; warp w takes row block I0 + w and
-// sweeps column blocks J0..J0+SYM_MACRO_COLS-1, skipping those below its row (the triangle) or
-// past the massive blocks.  Rows are written once per macro-tile, columns after the four warps' sums for
-// each column block are added in warp order through shared memory.
+// One CTA per macro-tile.  The macro-tile list entry is {system, first row block, first column block,
+// end of the system's massive blocks}; the CTA's rows are blocks I0 .. I0 + 3 and its columns J0 ..
+// J0 + SYM_MACRO_COLS - 1, without those below a row (the triangle) or past the massive blocks.  Rows
+// and columns are written once per macro-tile, summed over warps in warp order through shared memory.
+//
+// FP64 systems: sixteen warps; warp w takes row block I0 + w % 4 and a quarter, w / 4, of the steps of
+// each of its tiles, so that a system of a few blocks (one macro-tile per 128 x 64 bodies) still fills
+// the SM it runs on: the 1,000-body disk has 80 macro-tiles for 152 SMs.
 template <int MODE>
-__global__ void __launch_bounds__(128) k_trap_fp64(Dev D) {
-  __shared__ double colbuf[4][MC][3][32];     // [warp][column block][component][lane]
-  __shared__ JStage jstage[4];
+__global__ void __launch_bounds__(512) k_trap_df(Dev D) {
+  __shared__ ColDF col[MC][32];
+  __shared__ float4 cf[MC][32][2];              // kick 1: xf, yf, zf, vxf | vyf, vzf, lambda, sigma
+  __shared__ float2 rowbuf[16][3][32];          // [warp][component][lane]
+  __shared__ float2 colbuf[16][MC][3][32];
+  __shared__ int s_max[3];
+  __shared__ unsigned s_live[MC], s_mass[MC];
   __shared__ int s_item;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wr = w & 3, ws = w >> 2;
   const int nmac = D.ntiles_total;
   const int S = D.seg_len;
   int *counter = &D.work[MODE - 1];
+  float2 *part = reinterpret_cast<float2 *>(D.part);
   if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
+  if (threadIdx.x < 3) s_max[threadIdx.x] = 0;
   __syncthreads();
   int m0 = s_item * S;
   while (m0 < nmac) {
@@ -403,30 +432,81 @@ __global__ void __launch_bounds__(128) k_trap_fp64(Dev D) {
     for (int m = m0; m < m1; ++m) {
       const int4 mt = D.tiles[m];
       const TileCtx c = load_ctx(&D.disks[mt.x]);
-      const int I = mt.y + w;
+      // the grids: largest |x| of the macro-tile's live bodies, component by component
+      if (w < 4 + MC) {
+        const int b = w < 4 ? mt.y + w : mt.z + (w - 4);
+        const int p = b * 32 + lane;
+        const bool in = b < mt.w && p - c.off < c.n && D.alive[p];
+        const double *xs[3] = {D.x, D.y, D.z};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const unsigned hi = in ? (unsigned)__double2hiint(xs[k][p]) & 0x7FFFFFFFu : 0u;
+          const unsigned top = __reduce_max_sync(FULL, hi);
+          if (lane == 0) atomicMax(&s_max[k], (int)top);
+        }
+      }
+      __syncthreads();
+      const int E[3] = {grid_exp(s_max[0], c.kex), grid_exp(s_max[1], c.kex), grid_exp(s_max[2], c.kex)};
+      if (w >= 16 - MC) {                       // the last warps stage the column blocks
+        const int k = w - (16 - MC), b = mt.z + k, j = b * 32 + lane;
+        const bool in = b < mt.w, live = in && j - c.off < c.n && D.alive[j];
+        const unsigned ml = __ballot_sync(FULL, live), mm = __ballot_sync(FULL, live && j - c.off < c.nm);
+        if (lane == 0) { s_live[k] = ml; s_mass[k] = mm; }
+        if (in) {
+          float g[3][3];
+          const double p[3] = {D.x[j], D.y[j], D.z[j]};
+#pragma unroll
+          for (int q = 0; q < 3; ++q) on_grid(live ? p[q] : 0.0, E[q], c.kex, g[q][0], g[q][1], g[q][2]);
+          const df gm = split(scale2(D.gm[j], -c.keg));
+          col[k][lane].q[0] = make_float4(g[0][0], g[0][1], g[0][2], g[1][0]);
+          col[k][lane].q[1] = make_float4(g[1][1], g[1][2], g[2][0], g[2][1]);
+          col[k][lane].q[2] = make_float4(g[2][2], gm.h, gm.l, __int_as_float(MODE == 2 ? D.gid[j] : -1));
+          if (MODE == 1) {
+            cf[k][lane][0] = make_float4(D.xf[j], D.yf[j], D.zf[j], D.vxf[j]);
+            cf[k][lane][1] = make_float4(D.vyf[j], D.vzf[j], D.lamf[j], D.sigf[j]);
+          }
+        }
+      }
+      const int I = mt.y + wr;
       const bool has_row = I < mt.w;
-      RowF64 r;
-      if (has_row) row_load_fp64<MODE>(D, c, I, lane, r);
+      RowDF r;
+      if (has_row) row_load_df<MODE>(D, c, E, I, lane, r);
+      __syncthreads();
 #pragma unroll 1
       for (int k = 0; k < MC; ++k) {
         const int J = mt.z + k;
-        double cx = 0.0, cy = 0.0, cz = 0.0;
-        if (has_row && J < mt.w && J >= I)
-          tile_sweep_fp64<MODE>(D, c, mt.x, r, I, J, lane, &jstage[w], cx, cy, cz);
-        colbuf[w][k][0][lane] = cx; colbuf[w][k][1][lane] = cy; colbuf[w][k][2][lane] = cz;
-      }
-      double *rowp = D.part + part_row(m, w) + lane;
-      rowp[0] = has_row ? r.ax : 0.0; rowp[32] = has_row ? r.ay : 0.0; rowp[64] = has_row ? r.az : 0.0;
-      __syncthreads();
-      if (w < MC) {                                             // warp w adds column block w
-        double *colp = D.part + part_col(m, w) + lane;
+        if (has_row && J < mt.w && J >= I) {
+          const int q = I == J ? 4 : 8;         // a quarter of 16 or 32 steps
+          tile_steps_df<MODE>(D, c, mt.x, r, I, J, lane, q * ws, q * ws + q, col[k], cf[k], s_live[k], s_mass[k],
+                              colbuf[w][k]);
+        } else {
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-          colp[32 * q] = ((colbuf[0][w][q][lane] + colbuf[1][w][q][lane]) + colbuf[2][w][q][lane]) + colbuf[3][w][q][lane];
+          for (int q = 0; q < 3; ++q) colbuf[w][k][q][lane] = make_float2(0.0f, 0.0f);
+        }
       }
-      // the next item is taken while the columns are added (everyone has read s_item)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const df a = has_row ? renorm(r.acc[q]) : mk(0.0f, 0.0f);
+        rowbuf[w][q][lane] = make_float2(a.h, a.l);
+      }
+      // the next item is taken while the sums are formed (everyone has read s_item)
+      if (threadIdx.x < 3) s_max[threadIdx.x] = 0;
       if (m + 1 == m1 && threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-      __syncthreads();                        // colbuf is free, s_item is current
+      __syncthreads();
+      for (int i = threadIdx.x; i < SYM_MACRO_PART; i += 512) {     // [4 rows, MC columns][component][lane]
+        const int blk = i / 96, q = (i / 32) % 3, l = i & 31;
+        df a = mk(0.0f, 0.0f);
+        if (blk < 4) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v) accumulate(a, ld2(rowbuf[4 * v + blk][q][l]));
+        } else {
+#pragma unroll 4
+          for (int v = 0; v < 16; ++v) accumulate(a, ld2(colbuf[v][blk - 4][q][l]));
+        }
+        a = renorm(a);
+        part[(size_t)m * SYM_MACRO_PART + i] = make_float2(a.h, a.l);
+      }
+      __syncthreads();                          // the buffers are free
     }
     m0 = s_item * S;
   }
@@ -487,26 +567,34 @@ __global__ void __launch_bounds__(128) k_trap_mixed(Dev D) {
   }
 }
 
+// kick CTAs per multiprocessor a schedule may ask for
 int trap_blocks_per_sm(int precision) {
+  if (precision != SYMBA_PRECISION_MIXED) return 4;
   int nb = 0;
-  if (precision == SYMBA_PRECISION_MIXED) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trap_mixed<1>, 128, 0);
-    if (nb > 8) nb = 8;
-  } else {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trap_fp64<1>, 128, 0);
-    if (nb > 4) nb = 4;
-  }
-  return nb > 0 ? nb : 1;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trap_mixed<1>, 128, 0);
+  return nb > 8 ? 8 : (nb > 0 ? nb : 1);
 }
 
+// resident CTAs per multiprocessor, the schedule a pool starts with
+int trap_blocks_default(int precision) {
+  if (precision == SYMBA_PRECISION_MIXED) return trap_blocks_per_sm(precision);
+  int nb = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trap_df<1>, 512, 0);
+  return nb > 4 ? 4 : (nb > 0 ? nb : 1);
+}
+
+// No more CTAs than work items: with more, several on one SM could take an item each while other SMs
+// had none (80 macro-tiles of the 1,000-body disk for 608 CTAs).
 void launch_trap(const Dev &D, const LaunchCfg &L, int mode, int precision, cudaStream_t s) {
   if (D.ntiles_total <= 0) return;
+  const int items = (D.ntiles_total + D.seg_len - 1) / D.seg_len;
+  const int blocks = L.trap_blocks < items ? L.trap_blocks : items;
   if (precision == SYMBA_PRECISION_MIXED) {
-    if (mode == 1) k_trap_mixed<1><<<L.trap_blocks, 128, 0, s>>>(D);
-    else k_trap_mixed<2><<<L.trap_blocks, 128, 0, s>>>(D);
+    if (mode == 1) k_trap_mixed<1><<<blocks, 128, 0, s>>>(D);
+    else k_trap_mixed<2><<<blocks, 128, 0, s>>>(D);
   } else {
-    if (mode == 1) k_trap_fp64<1><<<L.trap_blocks, 128, 0, s>>>(D);
-    else k_trap_fp64<2><<<L.trap_blocks, 128, 0, s>>>(D);
+    if (mode == 1) k_trap_df<1><<<blocks, 512, 0, s>>>(D);
+    else k_trap_df<2><<<blocks, 512, 0, s>>>(D);
   }
 }
 
@@ -570,19 +658,25 @@ __device__ __forceinline__ double field_check(const Dev &D, const TileCtx &c, in
   return g0_weight(c, R0, __dsqrt_rn(er2));
 }
 
+// FP64 systems, in double-float as the tiles: one CTA per field block, its four warps each taking every
+// fourth chunk of 32 massive bodies; the four sums are added in warp order.
 template <int MODE>
-__global__ void __launch_bounds__(128) k_field_fp64(Dev D) {
-  __shared__ FieldSrc chunk[4][32];
+__global__ void __launch_bounds__(128) k_field_df(Dev D) {
+  __shared__ ColDF col[4][32];
+  __shared__ float4 cf[4][32][2];
+  __shared__ int sid[4][32];
+  __shared__ float2 sums[4][3][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int e = blockIdx.x * 4 + w;
-  if (e >= D.nfblk) return;
-  const int2 fb = D.fblk[e];                     // {system, global block}
+  const int2 fb = D.fblk[blockIdx.x];            // {system, global block}
   const TileCtx c = load_ctx(&D.disks[fb.x]);
-  FieldSrc *src = chunk[w];
   const int p = fb.y * 32 + lane;
   const int lp = p - c.off;
   const bool live = lp < c.n && D.alive[p];
-  const double xp = D.x[p], yp = D.y[p], zp = D.z[p];
+  const double xp[3] = {D.x[p], D.y[p], D.z[p]};
+  int top[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    top[k] = (int)__reduce_max_sync(FULL, live ? (unsigned)__double2hiint(xp[k]) & 0x7FFFFFFFu : 0u);
   const float xfp = D.xf[p], yfp = D.yf[p], zfp = D.zf[p];
   float vxfp = 0.f, vyfp = 0.f, vzfp = 0.f, lamp = 0.f, sigp = 0.f;
   int gidp = -1;
@@ -592,44 +686,81 @@ __global__ void __launch_bounds__(128) k_field_fp64(Dev D) {
     gidp = D.gid[p];
   }
   const float tauf = __double2float_ru(c.dt);
-  double ax = 0.0, ay = 0.0, az = 0.0;
-  for (int c0 = 0; c0 < c.nm; c0 += 32) {
+  df acc[3] = {mk(0.0f, 0.0f), mk(0.0f, 0.0f), mk(0.0f, 0.0f)};
+  for (int c0 = 32 * w; c0 < c.nm; c0 += 128) {
+    const int li = c0 + lane, j = c.off + li;
+    const bool ok = li < c.nm && D.alive[j];
+    const int jq = ok ? j : c.off;                // a valid address for the loads below
+    const double xj[3] = {D.x[jq], D.y[jq], D.z[jq]};
+    float g[3][3], gp[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int t = (int)__reduce_max_sync(FULL, ok ? (unsigned)__double2hiint(xj[k]) & 0x7FFFFFFFu : 0u);
+      const int E = grid_exp(max(t, top[k]), c.kex);
+      on_grid(ok ? xj[k] : 0.0, E, c.kex, g[k][0], g[k][1], g[k][2]);
+      on_grid(live ? xp[k] : 0.0, E, c.kex, gp[k][0], gp[k][1], gp[k][2]);
+    }
+    const df gm = split(scale2(D.gm[jq], -c.keg));
     __syncwarp();
-    stage_sources<MODE, false>(D, c, c0, lane, src);
+    col[w][lane].q[0] = make_float4(g[0][0], g[0][1], g[0][2], g[1][0]);
+    col[w][lane].q[1] = make_float4(g[1][1], g[1][2], g[2][0], g[2][1]);
+    col[w][lane].q[2] = make_float4(g[2][2], gm.h, gm.l, __int_as_float(MODE == 2 ? D.gid[jq] : -1));
+    sid[w][lane] = ok ? j : -1;
+    if (MODE == 1) {
+      cf[w][lane][0] = make_float4(D.xf[jq], D.yf[jq], D.zf[jq], D.vxf[jq]);
+      cf[w][lane][1] = make_float4(D.vyf[jq], D.vzf[jq], D.lamf[jq], D.sigf[jq]);
+    }
     __syncwarp();
     const int cnt = min(32, c.nm - c0);
 #pragma unroll 1
     for (int s = 0; s < cnt; ++s) {
-      const FieldSrc &q = src[s];
-      const bool valid = live && q.ok;
-      const double dx = q.x - xp, dy = q.y - yp, dz = q.z - zp;
-      const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      double sp = q.gm * rinv3(r2);
+      const float4 q0 = col[w][s].q[0], q1 = col[w][s].q[1], q2 = col[w][s].q[2];
+      const int id = sid[w][s];
+      const bool valid = live && id >= 0;
+      const df d[3] = {separation(q0.x, q0.y, q0.z, gp[0][0], gp[0][1], gp[0][2]),
+                       separation(q0.w, q1.x, q1.y, gp[1][0], gp[1][1], gp[1][2]),
+                       separation(q1.z, q1.w, q2.x, gp[2][0], gp[2][1], gp[2][2])};
+      df sp = mul(mk(q2.y, q2.z), inverse_cube(root(norm2(d))));
       if (MODE == 1) {
-        const float dxf = q.xf - xfp, dyf = q.yf - yfp, dzf = q.zf - zfp;
+        const float4 fa = cf[w][s][0], fq = cf[w][s][1];
+        const float dxf = fa.x - xfp, dyf = fa.y - yfp, dzf = fa.z - zfp;
         const float r2f = fmaf(dzf, dzf, fmaf(dyf, dyf, dxf * dxf));
-        const float dvxf = q.vxf - vxfp, dvyf = q.vyf - vyfp, dvzf = q.vzf - vzfp;
+        const float dvxf = fa.w - vxfp, dvyf = fq.x - vyfp, dvzf = fq.y - vzfp;
         const float vmag = sqrtf(fmaf(dvzf, dvzf, fmaf(dvyf, dvyf, dvxf * dvxf)));
-        const float Bf = fmaf(tauf, vmag, q.lam + lamp) * 1.0000039f + 1.9073486e-6f * (q.sig + sigp);
+        const float Bf = fmaf(tauf, vmag, fq.z + lamp) * 1.0000039f + 1.9073486e-6f * (fq.w + sigp);
         const bool cand = valid && !(r2f > Bf * Bf);
         if (__any_sync(FULL, cand)) {
-          if (cand) sp *= field_check(D, c, fb.x, q.id, p);
+          if (cand) {
+            const double wt = field_check(D, c, fb.x, id, p);
+            if (wt != 1.0) sp = weighted(sp, wt);
+          }
+          __syncwarp();
         }
-      } else if (gidp >= 0 && gidp == q.gid && valid) {
-        if (group_has_pair(D, gidp, q.id, p)) {
-          const double R0 = __dmul_rn(c.lam, __dadd_rn(D.rh[q.id], D.rh[p]));
-          sp *= g0_weight(c, R0, sqrt(r2));
+      } else if (gidp >= 0 && gidp == __float_as_int(q2.w) && valid) {
+        if (group_has_pair(D, gidp, id, p)) {
+          const double R0 = __dmul_rn(c.lam, __dadd_rn(D.rh[id], D.rh[p]));
+          const double ex = D.x[p] - D.x[id], ey = D.y[p] - D.y[id], ez = D.z[p] - D.z[id];
+          sp = weighted(sp, g0_weight(c, R0, sqrt(fma(ez, ez, fma(ey, ey, ex * ex)))));
         }
       }
-      sp = keep_or_zero(sp, valid);
-      ax = fma(sp, dx, ax); ay = fma(sp, dy, ay); az = fma(sp, dz, az);
+      sp.h = valid ? sp.h : 0.0f;
+      sp.l = valid ? sp.l : 0.0f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) accumulate(acc[k], mul(sp, d[k]));
     }
   }
-  if (live) {
-    const double h = 0.5 * c.dt;
-    D.vx[p] = __dadd_rn(D.vx[p], __dmul_rn(h, ax));
-    D.vy[p] = __dadd_rn(D.vy[p], __dmul_rn(h, ay));
-    D.vz[p] = __dadd_rn(D.vz[p], __dmul_rn(h, az));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const df a = renorm(acc[k]);
+    sums[w][k][lane] = make_float2(a.h, a.l);
+  }
+  __syncthreads();
+  if (w < 3 && live) {                           // warp w adds component w
+    df a = mk(0.0f, 0.0f);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) accumulate(a, ld2(sums[v][w][lane]));
+    double *vel = w == 0 ? D.vx : (w == 1 ? D.vy : D.vz);
+    vel[p] = __dadd_rn(vel[p], __dmul_rn(0.5 * c.dt, kick_value(a, c.keg - 2 * c.kex)));
   }
 }
 
@@ -705,12 +836,12 @@ __global__ void __launch_bounds__(128) k_field_mixed(Dev D) {
 
 void launch_field(const Dev &D, int mode, int precision, cudaStream_t s) {
   if (D.nfblk <= 0) return;
-  const int blocks = (D.nfblk + 3) / 4;
   if (precision == SYMBA_PRECISION_MIXED) {
+    const int blocks = (D.nfblk + 3) / 4;
     if (mode == 1) k_field_mixed<1><<<blocks, 128, 0, s>>>(D);
     else k_field_mixed<2><<<blocks, 128, 0, s>>>(D);
   } else {
-    if (mode == 1) k_field_fp64<1><<<blocks, 128, 0, s>>>(D);
-    else k_field_fp64<2><<<blocks, 128, 0, s>>>(D);
+    if (mode == 1) k_field_df<1><<<D.nfblk, 128, 0, s>>>(D);
+    else k_field_df<2><<<D.nfblk, 128, 0, s>>>(D);
   }
 }
