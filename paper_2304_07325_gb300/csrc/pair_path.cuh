@@ -36,8 +36,8 @@
 //     x' = x + h v - (u h^2/2) x,  v' = v - u h (1 - 3/2 p h) (x + h/2 v); 1/r^3 of the sun distance
 //     is carried along by the factor (1 + w)^(-3/2), w = 2 p h + q h^2 the relative change of r^2
 //     (|w| < 2e-6, formed in FP32 to 2^-43), and formed in full at every anchor;
-//   s < 5e-4: the Lagrange f and g series of drift_series() to order 6, 1/r^3, u, p and the leading
-//     coefficients in double-float; sub-steps with s > 2e-6 as 2 to 16 equal drifts;
+//   s <= 1.3e-4: the Lagrange f and g series of drift_series() to order 6, 1/r^3, u, p and the leading
+//     coefficients in double-float; sub-steps with s > 2e-6 as 4 to 16 equal drifts;
 //   longer intervals: the FP64 Kepler solver on the anchors.
 //
 // Cost and bound (one GB300 at 2.07 GHz).  A cleared order-2 sub-step is ~410 warp instructions, 95 %
@@ -188,7 +188,7 @@ __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int en
       m[c] = add_u(hn[c], mul(hk, d[c]));
       hv[c] = add(hv0[c], m[c]);
     }
-    const df_root q = root(norm2(xx));
+    const df_root q = root_fine(norm2(xx));
     const df ri2 = inverse(q);
     r3s = inverse_cube(q);
     ri2s = ri2.h;
@@ -349,7 +349,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
     df xx[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) xx[c] = add(x0[c], dl[c]);
-    const df_root q = root(norm2(xx));
+    const df_root q = root_fine(norm2(xx));
     r3s = inverse_cube(q);
     ri2s = q.t.h;
     fresh = true;
@@ -547,7 +547,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
     } else {
       plev = j - 1;
     }
-    if (__builtin_expect(so <= 5.1e-4f, 1)) {
+    if (__builtin_expect(so <= 1.28e-4f, 1)) {
       // ---- A run of sub-steps of level j by the series.  When the pair is between R_j and R_{j-1} it is
       // in F_{j-1} and not in F_j, and every level below j - 1 has weight zero there.  So when the M
       // sub-steps of level j are over, level j - 1 (and any that end with it) ends and starts again, and
@@ -556,7 +556,8 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
       // than M times h |dv| and what the kicks and the sun's tide can add to it; the sub-steps themselves
       // then have no decision left.  Without that clearance the run is this one sub-step.
       // Velocities and kicks here are times h / nq: a sub-step too long for the series (s > 2e-6) is taken
-      // as nq = 2 to 16 equal ones without a kick between them, which is the same motion.
+      // as nq = 4 to 16 equal ones of s <= 5e-7 without a kick between them, which is the same motion (the
+      // series' first omitted term, 1e-17 at s = 2e-6, is then added up 16 times).
       const float fM = (float)M;
       auto clear = [&](float speed, float u) {             // speed: h |dv| here; u: u h^2
         const float need = fM * (speed + fM * (kmax + 4.0f * fabsf(u) * Rp)) * 1.0001f;
@@ -567,7 +568,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
       substeps += end - 1 - cj;                            // (this one is counted)
       if (order2 && !fresh) sun();
       const bool wide = so >= 1e-8f;
-      const int nq = so <= 2.0e-6f ? 1 : (so <= 8.0e-6f ? 2 : (so <= 3.2e-5f ? 4 : (so <= 1.28e-4f ? 8 : 16)));
+      const int nq = so <= 2.0e-6f ? 1 : (so <= 8.0e-6f ? 4 : (so <= 3.2e-5f ? 8 : 16));   // s <= 5e-7 each
       const float fq = 1.0f / (float)nq;                   // a power of two: every scaling by it is exact
       const df hq = mk(fq * h.h, fq * h.l);
       const df g2 = ld(odd ? T->hb[j] : T->ha[j]);
