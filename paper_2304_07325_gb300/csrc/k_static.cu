@@ -13,6 +13,7 @@
 // SYMBA_ENERGY_STATIC_MAX_N = 65,534 (checked below at compile time).
 #include <algorithm>
 
+#include "energy.cuh"
 #include "internal.cuh"
 #include "ptr_class.h"
 
@@ -60,23 +61,28 @@ __global__ void __launch_bounds__(256) k_static_bodies(int n, const double *x, c
   for (int k = threadIdx.x; k < STATIC_ACCS * (SA_NDIG + 1); k += blockDim.x) (&s[0][0])[k] = 0ull;
   __syncthreads();
   const double Gm0 = __dmul_rn(G, m0);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double mi = m[i];
-    const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
-    const double ux = v[3 * i], uy = v[3 * i + 1], uz = v[3 * i + 2];
-    const double v2 = __dadd_rn(__dadd_rn(__dmul_rn(ux, ux), __dmul_rn(uy, uy)), __dmul_rn(uz, uz));
-    sa_add(s[0], __dmul_rn(__dmul_rn(0.5, mi), v2));
-    const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(px, px), __dmul_rn(py, py)), __dmul_rn(pz, pz)));
-    sa_add(s[0], -__ddiv_rn(__dmul_rn(Gm0, mi), r));
-    sa_add(s[1], __dmul_rn(mi, __dsub_rn(__dmul_rn(py, uz), __dmul_rn(pz, uy))));
-    sa_add(s[2], __dmul_rn(mi, __dsub_rn(__dmul_rn(pz, ux), __dmul_rn(px, uz))));
-    sa_add(s[3], __dmul_rn(mi, __dsub_rn(__dmul_rn(px, uy), __dmul_rn(py, ux))));
-    if (mi != 0.0) {
-      sa_add(s[4], __dmul_rn(mi, ux));
-      sa_add(s[5], __dmul_rn(mi, uy));
-      sa_add(s[6], __dmul_rn(mi, uz));
+  Window w[STATIC_ACCS];
+  for (int c = 0; c < STATIC_ACCS; ++c) win_clear(w[c]);
+  const int lane = threadIdx.x & 31;
+  // at most 65,534 / 32 iterations: far below WIN_TERMS
+  for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
+    const int i = i0 + lane;
+    double t[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, P[3] = {0.0, 0.0, 0.0};
+    if (i < n) {
+      const double mi = m[i];
+      const double ux = v[3 * i], uy = v[3 * i + 1], uz = v[3 * i + 2];
+      body_terms(mi, x[3 * i], x[3 * i + 1], x[3 * i + 2], ux, uy, uz, Gm0, t);
+      if (mi != 0.0) { P[0] = __dmul_rn(mi, ux); P[1] = __dmul_rn(mi, uy); P[2] = __dmul_rn(mi, uz); }
     }
+    win_add(w[0], s[0], t[0]);
+    win_add(w[0], s[0], t[1]);
+#pragma unroll
+    for (int c = 1; c < 4; ++c) win_add(w[c], s[c], t[c + 1]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) win_add(w[4 + c], s[4 + c], P[c]);
   }
+#pragma unroll
+  for (int c = 0; c < STATIC_ACCS; ++c) win_flush(w[c], s[c]);
   __syncthreads();
   for (int k = threadIdx.x; k < STATIC_ACCS * (SA_NDIG + 1); k += blockDim.x) {
     const unsigned long long val = (&s[0][0])[k];
@@ -95,21 +101,27 @@ __global__ void __launch_bounds__(256) k_static_pairs(int n, int nm, const doubl
   const long long nt = (long long)nbm * nb;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long t = warp; t < nt; t += nwarps) {
-    const int I = (int)(t / nb), J = (int)(t % nb);
+  const int cols = energy_cols(nt, nwarps), strips = 32 / cols;
+  Window w;
+  win_clear(w);
+  int terms = 0;
+  for (long long ts = warp; ts < nt * strips; ts += nwarps) {
+    const long long t = ts / strips;
+    const int I = (int)(t / nb), J = (int)(t % nb), c0 = (int)(ts % strips) * cols;
     if (J < I) continue;
-    const int i = I * 32 + lane;
-    if (i >= nm || i >= n) continue;
-    const double xi = x[3 * i], yi = x[3 * i + 1], zi = x[3 * i + 2];
-    const double Gmi = __dmul_rn(G, m[i]);
-    for (int k = 0; k < 32; ++k) {
+    const int i = I * 32 + lane, ic = min(i, n - 1);
+    const bool row = i < nm && i < n;
+    const double xi = x[3 * ic], yi = x[3 * ic + 1], zi = x[3 * ic + 2];
+    const double Gmi = __dmul_rn(G, m[ic]);
+    for (int k = c0; k < c0 + cols; ++k) {
       const int j = J * 32 + k;
-      if (j <= i || j >= n) continue;
-      const double dx = __dsub_rn(x[3 * j], xi), dy = __dsub_rn(x[3 * j + 1], yi), dz = __dsub_rn(x[3 * j + 2], zi);
-      const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
-      sa_add(s, -__ddiv_rn(__dmul_rn(Gmi, m[j]), r));
+      if (j >= n) break;
+      energy_pair(w, s, row && j > i, __dmul_rn(Gmi, m[j]), __dsub_rn(x[3 * j], xi),
+                  __dsub_rn(x[3 * j + 1], yi), __dsub_rn(x[3 * j + 2], zi));
     }
+    if ((terms += 32) == WIN_TERMS) { win_flush(w, s); terms = 0; }
   }
+  win_flush(w, s);
   __syncthreads();
   for (int k = threadIdx.x; k < SA_NDIG + 1; k += blockDim.x) {
     const unsigned long long val = s[k];
@@ -119,13 +131,19 @@ __global__ void __launch_bounds__(256) k_static_pairs(int n, int nm, const doubl
 
 // |P|^2 / (2 m0) with P rounded from its exact sums, then E, L rounded into out[0..3]
 __global__ void k_static_finish(double m0, unsigned long long *acc, double *out) {
-  if (threadIdx.x != 0) return;
-  const double Px = sa_round(acc + 4 * (SA_NDIG + 1));
-  const double Py = sa_round(acc + 5 * (SA_NDIG + 1));
-  const double Pz = sa_round(acc + 6 * (SA_NDIG + 1));
-  const double P2 = __dadd_rn(__dadd_rn(__dmul_rn(Px, Px), __dmul_rn(Py, Py)), __dmul_rn(Pz, Pz));
-  sa_add(acc, __ddiv_rn(P2, __dmul_rn(2.0, m0)));
-  for (int k = 0; k < 4; ++k) out[k] = sa_round(acc + k * (SA_NDIG + 1));
+  // each rounding is one thread's serial walk over the digits: side by side in the lanes
+  const int k = threadIdx.x;
+  double r = 0.0;
+  if (k >= 1 && k < STATIC_ACCS) r = sa_round(acc + k * (SA_NDIG + 1));
+  const double Px = __shfl_sync(0xffffffffu, r, 4);
+  const double Py = __shfl_sync(0xffffffffu, r, 5);
+  const double Pz = __shfl_sync(0xffffffffu, r, 6);
+  if (k == 0) {
+    const double P2 = __dadd_rn(__dadd_rn(__dmul_rn(Px, Px), __dmul_rn(Py, Py)), __dmul_rn(Pz, Pz));
+    sa_add(acc, __ddiv_rn(P2, __dmul_rn(2.0, m0)));
+    r = sa_round(acc);
+  }
+  if (k < 4) out[k] = r;
 }
 
 extern "C" int symba_energy_static(int n, int n_massive, const double *x, const double *v,
