@@ -188,7 +188,8 @@ void launch_prologue(const Dev &D, int ndisks, cudaStream_t s) { k_prologue<<<1,
 // exact total barycentric momentum P_d = sum m_i v_i of every system: MOM_CTAS CTAs per system
 // accumulate their share in the lanes' integer windows, join them in shared-memory digits, add the
 // digits to the system's global accumulator, and a second pass rounds it and clears it for the next
-// use.  (Straight into the digits, 32 lanes met at the same three: 24 -> 6 us a call.)
+// use.  (Straight into the digits, 32 lanes met at the same three: the accumulation took 29, 43 and
+// 64 us for 100, 1,000 and 10,000 bodies and takes 7, 8 and 11; the rounding after it takes 5 to 6.)
 // --------------------------------------------------------------------------------------------
 #define MOM_CTAS 24
 
