@@ -359,164 +359,6 @@ __device__ inline double sa_round(const unsigned long long *in) {
 }
 
 // --------------------------------------------------------------------------------------------
-// Kepler drift (Danby 1988, f and g functions): advance (x, v) by dt on the orbit of parameter
-// mu.  Elliptic orbits solve for the eccentric-anomaly difference X of
-//   X - ec sin X + es (1 - cos X) = n dt,  ec = 1 - r0/a, es = u / (n a^2)
-// with Danby's quartically convergent iteration from X = n dt, falling back to a bracketed
-// Newton-bisection; other orbits use universal variables with Stumpff functions.
-// Returns SYMBA_OK or SYMBA_E_KEPLER / SYMBA_E_NONFINITE.
-// --------------------------------------------------------------------------------------------
-__device__ inline void stumpff4(double z, double c[4]) {
-  if (fabs(z) < 0.1) {
-    for (int k = 0; k < 4; ++k) {
-      double term = 1.0, s = 0.0;
-      for (int i = 2; i <= k; ++i) term /= (double)i;
-      for (int j = 0; j < 24; ++j) {
-        s += term;
-        term *= -z / ((double)(2 * j + k + 1) * (double)(2 * j + k + 2));
-      }
-      c[k] = s;
-    }
-    return;
-  }
-  if (z > 0.0) {
-    const double sz = sqrt(z);
-    double sn, cs;
-    sincos(sz, &sn, &cs);
-    c[0] = cs;
-    c[1] = sn / sz;
-  } else {
-    const double sz = sqrt(-z);
-    c[0] = cosh(sz);
-    c[1] = sinh(sz) / sz;
-  }
-  c[2] = (1.0 - c[0]) / z;
-  c[3] = (1.0 - c[1]) / z;
-}
-
-// X - sin X = X^3 (1/3! - X^2/5! + X^4/7! - ...) in Horner form for |X| < 1/2 (through X^19,
-// the rest below 1e-21 relative), where the direct difference loses digits to cancellation
-__device__ inline double x_minus_sin(double X) {
-  if (fabs(X) >= 0.5) return X - sin(X);
-  const double z = X * X;
-  double p = -1.0 / 121645100408832000.0;                       // -1/19!
-  p = fma(p, z, 1.0 / 355687428096000.0);                       // 1/17!
-  p = fma(p, z, -1.0 / 1307674368000.0);                        // -1/15!
-  p = fma(p, z, 1.0 / 6227020800.0);                            // 1/13!
-  p = fma(p, z, -1.0 / 39916800.0);                             // -1/11!
-  p = fma(p, z, 1.0 / 362880.0);                                // 1/9!
-  p = fma(p, z, -1.0 / 5040.0);                                 // -1/7!
-  p = fma(p, z, 1.0 / 120.0);                                   // 1/5!
-  p = fma(p, z, -1.0 / 6.0);                                    // -1/3!
-  return -(X * z) * p;
-}
-
-// The new state is x0 + ((f - 1) x0 + g v0), v0 + (f' x0 + (g' - 1) v0): f - 1 and g' - 1 are
-// formed apart from the 1, which they would be rounded into when small.
-__device__ inline int kepler_drift(double mu, double dt, double &x, double &y, double &z,
-                                   double &vx, double &vy, double &vz) {
-  const double r0 = sqrt(fma(z, z, fma(y, y, x * x)));
-  const double v2 = fma(vz, vz, fma(vy, vy, vx * vx));
-  const double u = fma(z, vz, fma(y, vy, x * vx));
-  const double alpha = 2.0 * mu / r0 - v2;
-  if (!(r0 > 0.0) || !isfinite(alpha) || !isfinite(u)) return SYMBA_E_NONFINITE;
-  double fm1, g, fdot, gdm1;
-  if (alpha > 0.0) {
-    const double a = mu / alpha;
-    const double nn = sqrt(mu / (a * a * a));
-    const double ec = 1.0 - r0 / a;
-    const double es = u / (nn * a * a);
-    const double ndt = nn * dt;
-    double X = ndt, sx = 0.0, cx = 1.0;
-    bool ok = false;
-    for (int it = 0; it < 12; ++it) {
-      sincos(X, &sx, &cx);
-      const double omc = (cx > 0.0) ? sx * sx / (1.0 + cx) : 1.0 - cx;
-      const double F = X - ec * sx + es * omc - ndt;
-      const double Fp = 1.0 - ec * cx + es * sx;
-      const double Fpp = ec * sx + es * cx;
-      const double Fppp = ec * cx - es * sx;
-      const double d1 = -F / Fp;
-      const double d2 = -F / (Fp + 0.5 * d1 * Fpp);
-      const double d3 = -F / (Fp + 0.5 * d2 * Fpp + d2 * d2 * Fppp * (1.0 / 6.0));
-      X += d3;
-      if (fabs(d3) <= 1e-15 * fmax(1.0, fabs(X))) { ok = true; break; }
-    }
-    if (!ok) {
-      double lo = ndt - 2.5, hi = ndt + 2.5;
-      X = ndt;
-      for (int it = 0; it < 200; ++it) {
-        sincos(X, &sx, &cx);
-        const double omc = (cx > 0.0) ? sx * sx / (1.0 + cx) : 1.0 - cx;
-        const double F = X - ec * sx + es * omc - ndt;
-        const double Fp = 1.0 - ec * cx + es * sx;
-        if (F > 0.0) hi = X; else lo = X;
-        const double dX = -F / Fp;
-        double Xn = X + dX;
-        if (fabs(dX) <= 1e-15 * fmax(1.0, fabs(X))) { X = Xn; ok = true; break; }
-        if (!(Xn > lo && Xn < hi)) Xn = 0.5 * (lo + hi);
-        X = Xn;
-      }
-      if (!ok) return SYMBA_E_KEPLER;
-    }
-    sincos(X, &sx, &cx);
-    const double omc = (cx > 0.0) ? sx * sx / (1.0 + cx) : 1.0 - cx;
-    const double r = a * (1.0 - ec * cx + es * sx);
-    fm1 = -(a / r0) * omc;
-    g = dt - x_minus_sin(X) / nn;
-    fdot = -(a * a * nn * sx) / (r * r0);
-    gdm1 = -(a / r) * omc;
-  } else {
-    const double sgn = dt >= 0.0 ? 1.0 : -1.0;
-    double c[4];
-    double lo = 0.0, hi = fabs(dt) / r0;
-    if (hi == 0.0) return SYMBA_OK;
-    bool found = false;
-    for (int it = 0; it < 200; ++it) {
-      const double s = sgn * hi;
-      stumpff4(alpha * s * s, c);
-      const double F = r0 * s * c[1] + u * s * s * c[2] + mu * s * s * s * c[3] - dt;
-      if (sgn * F >= 0.0) { found = true; break; }
-      lo = hi;
-      hi *= 2.0;
-    }
-    if (!found) return SYMBA_E_KEPLER;
-    double sa = 0.5 * (lo + hi);
-    bool ok = false;
-    for (int it = 0; it < 400; ++it) {
-      const double s = sgn * sa;
-      stumpff4(alpha * s * s, c);
-      const double G1 = s * c[1], G2 = s * s * c[2], G3 = s * s * s * c[3];
-      const double F = r0 * G1 + u * G2 + mu * G3 - dt;
-      const double Fp = r0 * c[0] + u * G1 + mu * G2;
-      if (sgn * F > 0.0) hi = sa; else lo = sa;
-      const double ds = -F / Fp;
-      double sn = sa + sgn * ds;
-      if (fabs(ds) <= 1e-15 * fmax(1e-300, fabs(sa))) { sa = sn; ok = true; break; }
-      if (!(sn > lo && sn < hi)) sn = 0.5 * (lo + hi);
-      sa = sn;
-    }
-    if (!ok) return SYMBA_E_KEPLER;
-    const double s = sgn * sa;
-    stumpff4(alpha * s * s, c);
-    const double G1 = s * c[1], G2 = s * s * c[2], G3 = s * s * s * c[3];
-    const double r = r0 * c[0] + u * G1 + mu * G2;
-    fm1 = -mu * G2 / r0;
-    g = dt - mu * G3;
-    fdot = -mu * G1 / (r * r0);
-    gdm1 = -mu * G2 / r;
-  }
-  const double x0 = x, y0 = y, z0 = z, vx0 = vx, vy0 = vy, vz0 = vz;
-  x = x0 + fma(fm1, x0, g * vx0);
-  y = y0 + fma(fm1, y0, g * vy0);
-  z = z0 + fma(fm1, z0, g * vz0);
-  vx = vx0 + fma(gdm1, vx0, fdot * x0);
-  vy = vy0 + fma(gdm1, vy0, fdot * y0);
-  vz = vz0 + fma(gdm1, vz0, fdot * z0);
-  return SYMBA_OK;
-}
-
-// --------------------------------------------------------------------------------------------
 // Short-interval Kepler drift by the Lagrange f and g series (used on the deep recursion levels,
 // where the sub-step h is a tiny fraction of the orbit).  With u = mu/r^3, p = (x.v)/r^2,
 // q = v^2/r^2 - u, the derivatives of f and g obey f^(n+1) = (dA_n/dt - u B_n) f + (A_n + dB_n/dt) f'

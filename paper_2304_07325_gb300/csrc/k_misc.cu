@@ -3,6 +3,7 @@
 #include "df32.cuh"
 #include "energy.cuh"
 #include "internal.cuh"
+#include "kepler.cuh"
 
 // --------------------------------------------------------------------------------------------
 // per-system set-up: shell factors c_k = c_{k-1} / (R_k/R_{k+1}), c_0 = 1

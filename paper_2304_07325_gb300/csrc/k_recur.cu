@@ -29,6 +29,7 @@
 // The check below level 0 uses the division-free form of the predicate (same minimum-distance
 // test; identical except at exact ties).
 #include "internal.cuh"
+#include "kepler.cuh"
 
 #define FULL 0xffffffffu
 #define SMALL_M 32

@@ -254,6 +254,19 @@ __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int en
   S.ph = ph; S.qh = qh; S.uh = uh;
 }
 
+// The Kepler solver on a lane's anchors, called and not inlined: inlined, its registers are taken from
+// the sub-steps that never reach it.
+static __device__ __noinline__ int kepler_anchors(PairTab *T, int odd, double mu, double h) {
+  double x[3], v[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) { x[c] = T->X0[c][odd]; v[c] = T->V0[c][odd]; }
+  const int st = kepler_drift(mu, h, x[0], x[1], x[2], v[0], v[1], v[2]);
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) { T->X0[c][odd] = x[c]; T->V0[c][odd] = v[c]; }
+  return st;
+}
+
 // Runs the sub-steps of levels >= k with F_{k-1} = {q}, from the opening of a sub-step at level
 // k.  x, v: this lane's body (even lanes a, odd lanes b).  Returns 0 when level k has finished (k is
 // then k - 1), 1 when the pair may be in contact at the next check, or the scaled state does not
@@ -625,14 +638,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
 #pragma unroll
       for (int c = 0; c < 3; ++c) nu[c] = add(nu[c], mul(hc, d[c]));
       absorb();
-      double kx[3], kv[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) { kx[c] = T->X0[c][odd]; kv[c] = T->V0[c][odd]; }
-      const int st = kepler_drift(scale2(C.mu, -ea - 2 * eb), scale2(dp->hk[j], eb - ea), kx[0], kx[1], kx[2], kv[0],
-                                  kv[1], kv[2]);
-      __syncwarp();
-#pragma unroll
-      for (int c = 0; c < 3; ++c) { T->X0[c][odd] = kx[c]; T->V0[c][odd] = kv[c]; }
+      const int st = kepler_anchors(T, odd, scale2(C.mu, -ea - 2 * eb), scale2(dp->hk[j], eb - ea));
       if (st != SYMBA_OK && lane < 2) set_status(&D.stat[C.d], st);
       __syncwarp();
       order2 = false;
