@@ -13,7 +13,8 @@ LIB = os.path.join(OUT, "libsymba.so")
 SOURCES = ["api.cu", "k_misc.cu", "k_trap.cu", "k_groups.cu", "k_recur.cu", "k_static.cu", "k_tune.cu",
            "k_probe.cu"]
 HEADERS = [os.path.join(CSRC, "internal.cuh"), os.path.join(CSRC, "df32.cuh"), os.path.join(CSRC, "pair_path.cuh"),
-           os.path.join(CSRC, "energy.cuh"), os.path.join(CSRC, "kepler.cuh"),           os.path.join(CSRC, "ptr_class.h"),
+           os.path.join(CSRC, "energy.cuh"), os.path.join(CSRC, "kepler.cuh"),
+           os.path.join(CSRC, "group_path.cuh"),           os.path.join(CSRC, "ptr_class.h"),
            os.path.join(os.path.dirname(HERE), "include", "symba.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]

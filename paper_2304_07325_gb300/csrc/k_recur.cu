@@ -14,18 +14,19 @@
 //
 // The sub-step chain is latency-bound (GB300 issues one FP64 instruction per ~64 cycles per warp),
 // so it is kept short:
-//   - the group's bodies and pairs are gathered into a member-slot view that lives in shared
-//     memory for groups of up to 32 bodies and 64 pairs (global scratch otherwise), so phases
-//     exchange data through shared memory, and are scattered back at the end;
-//   - the deep-level drift uses the Lagrange f and g series when the sub-step is a tiny fraction
-//     of the orbit; square roots come from an integer-built FP32 seed plus one FP64 correction;
-//     the shell weights use per-level reciprocal tables;
-//   - the forces of the closing kick of one sub-step are reused by the opening kick of the next
-//     (same positions, same pairs, same weights);
+//   - a level whose F_{k-1} holds at most 32 pairs of at most 32 bodies runs in one warp's lanes, in
+//     double-float (group_path.cuh): small groups from level 1, larger ones from the level at which
+//     they have come down to that;
 //   - once F_{k-1} holds a single pair -- the close or bound pairs whose chains set the step
-//     time -- the sub-steps of levels >= k run in the single-pair path (pair_path.cuh), whose
-//     arithmetic is double-float.
-// Groups of at most 32 bodies and 32 pairs keep their state in registers (run_group_regs).
+//     time -- the sub-steps of levels >= k run in the single-pair path (pair_path.cuh);
+//   - the group's bodies and pairs are gathered into a member-slot view that lives in shared
+//     memory for groups of up to 32 bodies and 64 pairs (global scratch otherwise) and are scattered
+//     back at the end;
+//   - in the levels of larger sets, below, the drift uses the Lagrange f and g series when the sub-step
+//     is a tiny fraction of the orbit; square roots come from an integer-built FP32 seed plus one FP64
+//     correction; the shell weights use per-level reciprocal tables; the forces of the closing kick
+//     of one sub-step are reused by the opening kick of the next (same positions, pairs, weights).
+// A group whose quantities do not fit FP32's range in its own units stays in the FP64 levels below.
 // The check below level 0 uses the division-free form of the predicate (same minimum-distance
 // test; identical except at exact ties).
 #include "internal.cuh"
@@ -303,55 +304,40 @@ __device__ void drift_range(const GView &S, const GroupCtx &C, const Dev &D, int
 }
 
 #include "pair_path.cuh"
+#include "group_path.cuh"
+static_assert(sizeof(GroupTab) <= sizeof(SmallView::pf), "the table takes the force slots of a small view");
 
-__device__ void recurse(const GView &S, const GroupCtx &C, const Dev &D, const Levels &V, int lane, PairTab *T) {
+__device__ void recurse(const GView &S, const GroupCtx &C, const Dev &D, const Levels &V, int lane, const GroupScale &gs,
+                        PairTab *T, GroupTab *G) {
   int k = 1, deepest = 1, forces_at = -1;
   long long substeps = 0;
   V.h[1] = C.dt / (double)C.M;
   V.cnt[1] = 0;
   V.lenL[1] = C.pcnt;
   V.lenM[1] = C.mcnt;
-  bool start = true, aborted = false;
+  bool start = true, aborted = false, table = false;
   for (;;) {
     if (start) {
-      // a single pair below this level: the packed single-pair path
-      if (k >= 1 && C.l == 3 && V.lenL[k] == 1) {
-        const int q = S.perm[0];
-        const int a = S.pa[q], b = S.pb[q];
-        if (S.alive[a] && S.alive[b]) {
-          const int src = (lane & 1) ? b : a;
-          double px[3] = {S.x[src], S.y[src], S.z[src]}, pv[3] = {S.vx[src], S.vy[src], S.vz[src]};
-          const double R0 = S.R0[q], Rc = S.rad[a] + S.rad[b];
-          int plev = S.lev[q];
-          const int k0 = k;
-          __syncwarp();
-          const long long sub0 = substeps;
-          const int rc = pair_run(D, C, lane, V.h, V.cnt, T, px, pv, S.gm[a], S.gm[b], R0 * R0,
-                                  S.invR0[q], 1.0000001 * (Rc * Rc), k, plev, substeps, deepest);
-          if (lane == 0) atomicAdd(&D.stat[C.d].pair_substeps, (unsigned long long)(substeps - sub0));
-          if (lane < 2) {
-            S.x[src] = px[0]; S.y[src] = px[1]; S.z[src] = px[2];
-            S.vx[src] = pv[0]; S.vy[src] = pv[1]; S.vz[src] = pv[2];
-          }
-          if (lane == 0) S.lev[q] = plev;
-          // levels entered below k0 hold the same single pair and its two bodies
-          for (int i = k0 + 1 + lane; i <= k; i += 32) { V.lenL[i] = 1; V.lenM[i] = V.lenM[k0]; }
-          __syncwarp();
-          forces_at = -1;
-          if (rc == 0) {
-            if (k == 0) break;
-            start = false;
-            continue;
-          }
-          if (rc == 2) { aborted = true; break; }
-        }
+      // few enough pairs and bodies for one warp's lanes: levels >= k in group_path.cuh
+      if (gs.fits && V.lenL[k] <= 32 && V.lenM[k] <= 32) {
+        if (!table) group_table(G, C, gs, lane);
+        table = true;
+        bool merged = false;
+        aborted = !small_levels(D, C, S, gs, lane, V.lenM[k], V.lenL[k], V.h, V.cnt, T, G, k, substeps, deepest, &merged);
+        if (aborted || --k == 0) break;
+        if (merged)
+          for (int q = lane; q < C.pcnt; q += 32) set_r0(S, C, q);
+        __syncwarp();
+        forces_at = -1;
+        start = false;
+        continue;
       }
       ++substeps;
       if (substeps > C.max_substeps) { aborted = true; break; }
       deepest = max(deepest, k);
       bool merged = false;
       const bool fk = check_level(S, C, D, V, k, lane, &merged);
-      if (merged || forces_at != k) { forces_level(S, C, V, k, lane); forces_at = k; }
+      if (merged || forces_at != k) { forces_level(S, C, V, k, lane); forces_at = k; table = false; }
       kick_level(S, V, k, 0.5 * V.h[k], lane);
       const bool deeper = fk && (k + 1 <= C.max_depth);
       if (fk && !deeper && lane == 0) set_status(&D.stat[C.d], SYMBA_E_DEPTH);
@@ -381,6 +367,7 @@ __device__ void recurse(const GView &S, const GroupCtx &C, const Dev &D, const L
     // (iv) of E_k, then the next of its M calls or back to the parent's (iv)
     forces_level(S, C, V, k, lane);
     forces_at = k;
+    table = false;                         // (the table may lie where a small view keeps its forces)
     kick_level(S, V, k, 0.5 * V.h[k], lane);
     if (++V.cnt[k] < C.M) { start = true; continue; }
     --k;
@@ -395,280 +382,7 @@ __device__ void recurse(const GView &S, const GroupCtx &C, const Dev &D, const L
   }
 }
 
-// --------------------------------------------------------------------------------------------
-// Register-resident path for groups of at most 32 bodies and 32 pairs: lane a holds body a, lane
-// q holds pair q (member slots, critical radius, level mark, the last forces).  Pairs read their
-// bodies with warp shuffles; F_{k-1} and F_k are ballot masks, a body's pairs a bitmask, so no
-// list is stored or partitioned.  Same method, same order of accumulation (pair-list order).
-// --------------------------------------------------------------------------------------------
-#define SH(v, src) __shfl_sync(FULL, (v), (src))
-
-__device__ __forceinline__ bool contact_regs(double xa, double ya, double za, double xb, double yb,
-                                             double zb, double ra, double rb) {
-  const double dx = __dsub_rn(xb, xa), dy = __dsub_rn(yb, ya), dz = __dsub_rn(zb, za);
-  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-  const double Rc = __dadd_rn(ra, rb);
-  return r2 < __dmul_rn(Rc, Rc);
-}
-
-__device__ __forceinline__ bool predicate_regs(double dx, double dy, double dz, double r2, double dvx,
-                                               double dvy, double dvz, double R2, double h) {
-  if (lt_nn(r2, R2)) return true;
-  const double vr = fma(dz, dvz, fma(dy, dvy, dx * dvx));
-  if (!is_neg(vr)) return false;
-  const double v2 = fma(dvz, dvz, fma(dvy, dvy, dvx * dvx));
-  if (lt_nn(neg(vr), h * v2)) return lt_nn(fma(r2, v2, -vr * vr), R2 * v2);
-  const double e = fma(h, fma(h, v2, 2.0 * vr), r2);
-  return is_neg(e) || lt_nn(e, R2);
-}
-
-__device__ void run_group_regs(const Dev &D, const GroupCtx &C, int lane, double *hs, int *cs, PairTab *T) {
-  const int nm = C.mcnt, np = C.pcnt;
-  const bool ism = lane < nm, isp = lane < np;
-  // bodies
-  int pglob = -1;
-  double x = 0.0, y = 0.0, z = 0.0, vx = 0.0, vy = 0.0, vz = 0.0, m = 0.0, gm = 0.0, rad = 0.0, rh = 0.0;
-  int alive = 0;
-  if (ism) {
-    pglob = D.gmem[C.moff + lane];
-    x = D.x[pglob]; y = D.y[pglob]; z = D.z[pglob];
-    vx = D.vx[pglob]; vy = D.vy[pglob]; vz = D.vz[pglob];
-    m = D.m[pglob]; gm = D.gm[pglob]; rad = D.rad[pglob]; rh = D.rh[pglob];
-    alive = D.alive[pglob];
-    D.mslot[pglob] = lane;
-  }
-  __syncwarp();
-  // pairs
-  int ia = 0, ib = 0, lev = -1;
-  if (isp) {
-    ia = D.mslot[D.gpi[C.poff + lane]];
-    ib = D.mslot[D.gpj[C.poff + lane]];
-    lev = 0;
-  }
-  // per-pair constants: critical radius R_0, 1/R_0, R_0^2 and the contact prefilter threshold
-  double R0, iR0, R0sq, Rcut;
-  auto pair_consts = [&]() {
-    const double ra = SH(rh, ia), rb = SH(rh, ib);
-    const double sa = SH(rad, ia), sb = SH(rad, ib);
-    R0 = __dmul_rn(C.lam, __dadd_rn(ra, rb));
-    iR0 = R0 > 0.0 ? 1.0 / R0 : 0.0;
-    R0sq = R0 * R0;
-    const double Rc = sa + sb;
-    Rcut = 1.0000001 * (Rc * Rc);
-  };
-  pair_consts();
-  unsigned im = 0u, jm = 0u;
-  for (int q = 0; q < np; ++q) {
-    const int a_ = SH(ia, q), b_ = SH(ib, q);
-    if (a_ == lane) im |= 1u << q;
-    if (b_ == lane) jm |= 1u << q;
-  }
-  const unsigned adjm = ism ? (im | jm) : 0u;
-  double fdx = 0.0, fdy = 0.0, fdz = 0.0, ffi = 0.0, ffj = 0.0;   // forces of pair `lane`
-
-  auto forces = [&](int k) {
-    const unsigned Lm = __ballot_sync(FULL, isp && lev >= k - 1);
-    const double xa = SH(x, ia), ya = SH(y, ia), za = SH(z, ia);
-    const double xb = SH(x, ib), yb = SH(y, ib), zb = SH(z, ib);
-    const double ga = SH(gm, ia), gb = SH(gm, ib);
-    const int aa = SH(alive, ia), ab = SH(alive, ib);
-    fdx = fdy = fdz = ffi = ffj = 0.0;
-    if (((Lm >> lane) & 1u) && aa && ab) {
-      fdx = xb - xa; fdy = yb - ya; fdz = zb - za;
-      const double r2 = fma(fdz, fdz, fma(fdy, fdy, fdx * fdx));
-      const double ri = rsqrt_fp64(r2);
-      const double rho = r2 * ri * iR0;
-      const double ck = C.dp->ck[k], ck1 = C.dp->ck[k + 1];
-      double w;
-      if (k == 0 || lt_nn(rho, ck)) w = partition_fn((rho - ck1) * C.dp->invdc[k], C.l);
-      else w = 1.0 - partition_fn((rho - ck) * C.dp->invdc[k - 1], C.l);
-      const double s = w * (ri * ri * ri);
-      ffi = gb * s;
-      ffj = ga * s;
-    }
-  };
-
-  auto kick = [&](int k, double hh) {
-    const unsigned Lm = __ballot_sync(FULL, isp && lev >= k - 1);
-    unsigned mine = adjm & Lm;
-    const bool inS = mine != 0u;
-    const int iters = __reduce_max_sync(FULL, (unsigned)__popc(mine));
-    double ax = 0.0, ay = 0.0, az = 0.0;
-    for (int it = 0; it < iters; ++it) {
-      const int q = mine ? (__ffs(mine) - 1) : lane;
-      const double qx = SH(fdx, q), qy = SH(fdy, q), qz = SH(fdz, q), qi = SH(ffi, q), qj = SH(ffj, q);
-      if (mine) {
-        const double f = ((im >> q) & 1u) ? qi : -qj;
-        ax = fma(f, qx, ax); ay = fma(f, qy, ay); az = fma(f, qz, az);
-        mine &= mine - 1u;
-      }
-    }
-    if (inS && alive) {
-      vx = fma(hh, ax, vx); vy = fma(hh, ay, vy); vz = fma(hh, az, vz);
-    }
-  };
-
-  auto drift = [&](int k, double h, bool all) {
-    const unsigned Lm = __ballot_sync(FULL, isp && lev >= k - 1);
-    const unsigned Fm = __ballot_sync(FULL, isp && lev >= k);
-    const bool inS = (adjm & Lm) != 0u, inF = (adjm & Fm) != 0u;
-    if (alive && inS && (all || !inF)) {
-      if (!drift_series(C.mu, h, x, y, z, vx, vy, vz)) {
-        const int st = kepler_drift(C.mu, h, x, y, z, vx, vy, vz);
-        if (st != SYMBA_OK) set_status(&D.stat[C.d], st);
-      }
-    }
-  };
-
-  // (i): returns whether F_k is non-empty; *merged when bodies merged
-  auto check = [&](int k, double h, bool *merged) -> bool {
-    const bool inL = isp && lev >= k - 1;
-    const double xa = SH(x, ia), ya = SH(y, ia), za = SH(z, ia);
-    const double xb = SH(x, ib), yb = SH(y, ib), zb = SH(z, ib);
-    const int aa = SH(alive, ia), ab = SH(alive, ib);
-    const double dx = xb - xa, dy = yb - ya, dz = zb - za;
-    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const bool both = inL && aa && ab;
-    const double rda = SH(rad, ia), rdb = SH(rad, ib);
-    const bool ct = both && lt_nn(r2, Rcut) && contact_regs(xa, ya, za, xb, yb, zb, rda, rdb);
-    if (!__any_sync(FULL, ct)) {
-      const double vxa = SH(vx, ia), vya = SH(vy, ia), vza = SH(vz, ia);
-      const double vxb = SH(vx, ib), vyb = SH(vy, ib), vzb = SH(vz, ib);
-      bool fl = false;
-      if (both) fl = predicate_regs(dx, dy, dz, r2, vxb - vxa, vyb - vya, vzb - vza, R0sq * C.dp->ck2[k], h);
-      if (inL) lev = fl ? k : k - 1;
-      *merged = false;
-      return __any_sync(FULL, fl) != 0;
-    }
-    // mergers: the pairs one by one in list order, every lane following the same sequence
-    bool nonempty = false;
-    for (int q = 0; q < np; ++q) {
-      if (SH(lev, q) < k - 1) continue;
-      const int a_ = SH(ia, q), b_ = SH(ib, q);
-      bool fl = false;
-      if (SH(alive, a_) && SH(alive, b_)) {
-        const double xa_ = SH(x, a_), ya_ = SH(y, a_), za_ = SH(z, a_);
-        const double xb_ = SH(x, b_), yb_ = SH(y, b_), zb_ = SH(z, b_);
-        const double ra_ = SH(rad, a_), rb_ = SH(rad, b_);
-        const double vxa_ = SH(vx, a_), vya_ = SH(vy, a_), vza_ = SH(vz, a_);
-        const double vxb_ = SH(vx, b_), vyb_ = SH(vy, b_), vzb_ = SH(vz, b_);
-        const double ma = SH(m, a_), mb = SH(m, b_), rha = SH(rh, a_);
-        if (contact_regs(xa_, ya_, za_, xb_, yb_, zb_, ra_, rb_)) {
-          const double Mt = __dadd_rn(ma, mb);
-          if (lane == a_) {
-            if (Mt > 0.0) {
-              x = __ddiv_rn(__dadd_rn(__dmul_rn(ma, xa_), __dmul_rn(mb, xb_)), Mt);
-              y = __ddiv_rn(__dadd_rn(__dmul_rn(ma, ya_), __dmul_rn(mb, yb_)), Mt);
-              z = __ddiv_rn(__dadd_rn(__dmul_rn(ma, za_), __dmul_rn(mb, zb_)), Mt);
-              vx = __ddiv_rn(__dadd_rn(__dmul_rn(ma, vxa_), __dmul_rn(mb, vxb_)), Mt);
-              vy = __ddiv_rn(__dadd_rn(__dmul_rn(ma, vya_), __dmul_rn(mb, vyb_)), Mt);
-              vz = __ddiv_rn(__dadd_rn(__dmul_rn(ma, vza_), __dmul_rn(mb, vzb_)), Mt);
-            }
-            rad = cbrt_rn(__dadd_rn(__dmul_rn(__dmul_rn(ra_, ra_), ra_), __dmul_rn(__dmul_rn(rb_, rb_), rb_)));
-            if (ma > 0.0) rh = __dmul_rn(rha, cbrt_rn(__ddiv_rn(Mt, ma)));
-            m = Mt;
-            gm = __dmul_rn(C.G, Mt);
-          }
-          if (lane == b_) { m = 0.0; gm = 0.0; rad = 0.0; rh = 0.0; alive = 0; }
-          if (lane == 0) atomicAdd(&D.stat[C.d].merges, 1ull);
-          // critical radii and contact thresholds follow the new body
-          pair_consts();
-        } else {
-          const double R0q = SH(R0, q);
-          fl = predicate_regs(xb_ - xa_, yb_ - ya_, zb_ - za_,
-                              fma(zb_ - za_, zb_ - za_, fma(yb_ - ya_, yb_ - ya_, (xb_ - xa_) * (xb_ - xa_))),
-                              vxb_ - vxa_, vyb_ - vya_, vzb_ - vza_, R0q * R0q * C.dp->ck2[k], h);
-        }
-      }
-      if (lane == q) lev = fl ? k : k - 1;
-      nonempty |= fl;
-    }
-    *merged = true;
-    return nonempty;
-  };
-
-  int k = 1, deepest = 1, forces_at = -1;
-  long long substeps = 0;
-  hs[1] = C.dt / (double)C.M;
-  cs[1] = 0;
-  bool start = true, aborted = false;
-  for (;;) {
-    if (start) {
-      // a single pair below this level: the packed single-pair path
-      if (k >= 1 && C.l == 3) {
-        const unsigned Lm = __ballot_sync(FULL, isp && lev >= k - 1);
-        if (__popc(Lm) == 1) {
-          const int q = __ffs(Lm) - 1;
-          const int a_ = SH(ia, q), b_ = SH(ib, q);
-          if (SH(alive, a_) && SH(alive, b_)) {
-            const int src = (lane & 1) ? b_ : a_;
-            double px[3] = {SH(x, src), SH(y, src), SH(z, src)}, pv[3] = {SH(vx, src), SH(vy, src), SH(vz, src)};
-            int plev = SH(lev, q);
-            const long long sub0 = substeps;
-            const int rc = pair_run(D, C, lane, hs, cs, T, px, pv, SH(gm, a_), SH(gm, b_), SH(R0sq, q),
-                                    SH(iR0, q), SH(Rcut, q), k, plev, substeps, deepest);
-            if (lane == 0) atomicAdd(&D.stat[C.d].pair_substeps, (unsigned long long)(substeps - sub0));
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const double xa_ = SH(px[c], 0), xb_ = SH(px[c], 1), va_ = SH(pv[c], 0), vb_ = SH(pv[c], 1);
-              double &X_ = c == 0 ? x : (c == 1 ? y : z), &V_ = c == 0 ? vx : (c == 1 ? vy : vz);
-              if (lane == a_) { X_ = xa_; V_ = va_; }
-              if (lane == b_) { X_ = xb_; V_ = vb_; }
-            }
-            if (lane == q) lev = plev;
-            forces_at = -1;
-            if (rc == 0) {            // level k + 1 finished: continue with the closing kick of k
-              if (k == 0) break;
-              start = false;
-              continue;
-            }
-            if (rc == 2) { aborted = true; break; }
-            // rc == 1: a contact may be due; this sub-step takes the general path
-          }
-        }
-      }
-      ++substeps;
-      if (substeps > C.max_substeps) { aborted = true; break; }
-      deepest = max(deepest, k);
-      bool merged = false;
-      const bool fk = check(k, hs[k], &merged);
-      if (merged || forces_at != k) { forces(k); forces_at = k; }
-      kick(k, 0.5 * hs[k]);
-      const bool deeper = fk && (k + 1 <= C.max_depth);
-      if (fk && !deeper && lane == 0) set_status(&D.stat[C.d], SYMBA_E_DEPTH);
-      drift(k, hs[k], fk && !deeper);
-      if (deeper) {
-        ++k;
-        hs[k] = sub_interval(C, hs[k - 1]);
-        cs[k] = 0;
-        continue;
-      }
-      start = false;
-    }
-    forces(k);
-    forces_at = k;
-    kick(k, 0.5 * hs[k]);
-    if (++cs[k] < C.M) { start = true; continue; }
-    --k;
-    forces_at = -1;
-    if (k == 0) break;
-  }
-  if (aborted && lane == 0) set_status(&D.stat[C.d], SYMBA_E_DEPTH);
-  if (lane == 0) {
-    atomicMax(&D.stat[C.d].max_depth, deepest);
-    atomicAdd(&D.stat[C.d].substeps, (unsigned long long)substeps);
-    atomicMax(&D.stat[C.d].max_chain, (unsigned long long)substeps);
-  }
-  if (ism) {
-    D.x[pglob] = x; D.y[pglob] = y; D.z[pglob] = z;
-    D.vx[pglob] = vx; D.vy[pglob] = vy; D.vz[pglob] = vz;
-    D.m[pglob] = m; D.gm[pglob] = gm; D.rad[pglob] = rad; D.rh[pglob] = rh;
-    D.alive[pglob] = alive;
-  }
-  __syncwarp();
-}
-
-__device__ void run_group(const Dev &D, int g, int lane, const Levels &V, SmallView *sv, PairTab *T) {
+__device__ void run_group(const Dev &D, int g, int lane, const Levels &V, SmallView *sv, GView &S, PairTab *T) {
   GroupCtx C;
   C.moff = D.g_moff[g];
   C.mcnt = D.g_mcnt[g];
@@ -681,11 +395,6 @@ __device__ void run_group(const Dev &D, int g, int lane, const Levels &V, SmallV
   C.mu = __dmul_rn(C.dp->G, C.dp->m0);
   C.invM = 1.0 / (double)C.M;
 
-  if (C.mcnt <= 32 && C.pcnt <= 32) {
-    run_group_regs(D, C, lane, V.h, V.cnt, T);
-    return;
-  }
-  GView S;
   const bool small = C.mcnt <= SMALL_M && C.pcnt <= SMALL_P;
   if (small) {
     S.x = sv->x; S.y = sv->y; S.z = sv->z; S.vx = sv->vx; S.vy = sv->vy; S.vz = sv->vz;
@@ -723,7 +432,9 @@ __device__ void run_group(const Dev &D, int g, int lane, const Levels &V, SmallV
   }
   __syncwarp();
   for (int q = lane; q < C.pcnt; q += 32) set_r0(S, C, q);
-  if (lane == 0) {
+  __syncwarp();
+  const GroupScale gs = group_scale(S, C, lane);
+  if (lane == 0 && !(gs.fits && C.mcnt <= 32 && C.pcnt <= 32)) {
     int o = 0;
     for (int q = 0; q < C.pcnt; ++q) { S.adj_cnt[S.pa[q]]++; S.adj_cnt[S.pb[q]]++; }
     for (int a = 0; a < C.mcnt; ++a) { S.adj_off[a] = o; o += S.adj_cnt[a]; S.adj_cnt[a] = 0; }
@@ -735,7 +446,7 @@ __device__ void run_group(const Dev &D, int g, int lane, const Levels &V, SmallV
   }
   __syncwarp();
 
-  recurse(S, C, D, V, lane, T);
+  recurse(S, C, D, V, lane, gs, T, (GroupTab *)sv->pf);
 
   // scatter back
   for (int a = lane; a < C.mcnt; a += 32) {
@@ -753,6 +464,7 @@ __global__ void __launch_bounds__(128) k_recursion(Dev D) {
   __shared__ int cs[4][SYM_MAX_LEVELS + 2], ls[4][SYM_MAX_LEVELS + 2], ms[4][SYM_MAX_LEVELS + 2];
   __shared__ SmallView sview[4];
   __shared__ PairTab ptab[4];
+  __shared__ GView views[4];              // (24 pointers: registers the sub-steps need)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const Levels V{hs[w], cs[w], ls[w], ms[w]};
   const int total = *D.rec_total;
@@ -761,7 +473,7 @@ __global__ void __launch_bounds__(128) k_recursion(Dev D) {
     if (lane == 0) item = atomicAdd(&D.work[2], 1);
     item = __shfl_sync(FULL, item, 0);
     if (item >= total) break;
-    run_group(D, D.rec_items[item], lane, V, &sview[w], &ptab[w]);
+    run_group(D, D.rec_items[item], lane, V, &sview[w], views[w], &ptab[w]);
   }
 }
 

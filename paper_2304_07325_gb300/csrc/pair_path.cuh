@@ -54,18 +54,23 @@
 
 #define ANCHOR_N 128         // sub-steps between anchors
 
-// per-level constants of one pair, in the scaled units (shared memory, one per warp)
-struct PairTab {
+// per-level constants of a group in its scaled units (shared memory, one per warp)
+struct GroupTab {
   float2 h[SYM_MAX_LEVELS + 2];    // sub-step h_j
+  float2 rh[SYM_MAX_LEVELS + 2];   // 1 / h_j
   float2 mh[SYM_MAX_LEVELS + 2];   // mu h_j^2
+  float2 A[SYM_MAX_LEVELS + 2];    // argument of g_j about the middle of its zone: y = A r/R_0 + B =
+  float2 B[SYM_MAX_LEVELS + 2];    // 2 (r - R_{j+1}) / (R_j - R_{j+1}) - 1
+  float2 c2[SYM_MAX_LEVELS + 2];   // (R_j / R_0)^2
+};
+// and those of one pair
+struct PairTab {
   float2 ga[SYM_MAX_LEVELS + 2];   // G m_b h_j / 2, the kick's factor on body a
   float2 gb[SYM_MAX_LEVELS + 2];   // G m_a h_j / 2, on body b
   float2 ha[SYM_MAX_LEVELS + 2];   // h_j times the same
   float2 hb[SYM_MAX_LEVELS + 2];
   float2 R2[SYM_MAX_LEVELS + 2];   // R_j^2
-  float2 A[SYM_MAX_LEVELS + 2];    // argument of g_j about the middle of its zone: y = r A + B =
-  float2 B[SYM_MAX_LEVELS + 2];    // 2 (r - R_{j+1}) / (R_j - R_{j+1}) - 1
-  float2 rh[SYM_MAX_LEVELS + 2];   // 1 / h_j
+  float2 A[SYM_MAX_LEVELS + 2];    // A of the group's table over R_0
   double X0[3][2], V0[3][2];       // the anchors of bodies a, b
 };
 __device__ __forceinline__ df ld(const float2 &v) { return mk(v.x, v.y); }
@@ -164,6 +169,68 @@ __device__ __forceinline__ void run_order2(Run &S, df gh, df mhh, int cj, int en
   S.ph = ph; S.qh = qh; S.uh = uh;
 }
 
+// The Lagrange f and g series of drift_series() to order 6 at position xx with velocity hv / h: increments
+// dx of the position and dv / h of the velocity.  mhh: mu h^2.
+struct Series {
+  df r3s;                          // 1/r^3 from the sun
+  float ri2s, P, Q, U;             // 1/r^2, p h, q h^2, u h^2
+};
+__device__ __forceinline__ Series series_increments(const df (&xx)[3], const df (&hv)[3], df mhh, bool wide,
+                                                    df (&dx)[3], df (&dv)[3]) {
+  // its coefficients over u h^2 (drift_series()) are FP32 where what they multiply is below 1e-12:
+  // their error, unlike a rounding of x or v, is the same from one sub-step to the next and adds up.
+  // With s > 1e-8 (wide) that leaves out c4 in f' and g - h.
+  Series o;
+  const df_root q = root_fine(norm2(xx));
+  const df ri2 = inverse(q);
+  o.r3s = inverse_cube(q);
+  o.ri2s = ri2.h;
+  const df u = renorm(mul(mhh, o.r3s));                        // u h^2
+  const df pd = renorm(mul(dot3(xx, hv), ri2));              // p h
+  const float U = u.h, P = pd.h, P2 = P * P;
+  float Q;                                                   // q h^2
+  df c4d;                                                    // 4 c4 / (u h^2)
+  if (wide) {
+    const df qd = add(mul(norm2(hv), ri2), neg(u));
+    Q = qd.h;
+    c4d = mul(add(add(mul(qd, 3.0f), u), mul(sqr(pd), -15.0f)), mk(0.16666667f, -4.967054e-09f));
+  } else {
+    Q = fmaf(fmaf(hv[2].h, hv[2].h, fmaf(hv[1].h, hv[1].h, hv[0].h * hv[0].h)), ri2.h, -U);
+    c4d = mk((3.0f * Q - 15.0f * P2 + U) * (1.0f / 6.0f), 0.0f);
+  }
+  const float c4 = 0.25f * c4d.h;
+  const float c5 = P * (7.0f * P2 - 3.0f * Q - U) * 0.125f;
+  const float c6 = (P2 * (-945.0f * P2 + 630.0f * Q + 210.0f * U) - 45.0f * Q * Q - 24.0f * U * Q - U * U) *
+                   (1.0f / 720.0f);
+  const float d5 = (9.0f * Q - 45.0f * P2 + U) * (1.0f / 120.0f);
+  const float d6 = P * (14.0f * P2 - 6.0f * Q - U) * (1.0f / 24.0f);
+  // f - 1 = (u h^2/2) (-1 + p h + ...), h f' = u h^2 (-1 + 3/2 p h + ...), g' - 1 = (u h^2/2)
+  // (-1 + 2 p h + ...), g - h = h (u h^2/6) (-1 + 3/2 p h + ...)
+  auto bracket = [&](float k, float rest, float rest_l) {
+    const df p = mul(pd, k), t = fast_two_sum(-1.0f, p.h), b = fast_two_sum(t.h, rest);
+    return mk(b.h, __fadd_rn(__fadd_rn(b.l, t.l), __fadd_rn(p.l, rest_l)));
+  };
+  const df u2 = mk(0.5f * u.h, 0.5f * u.l);
+  const df fm1 = mul(u2, bracket(1.0f, 2.0f * (c4 + c5 + c6), 0.0f));
+  const df fd = mul(u, bracket(1.5f, c4d.h, c4d.l + (5.0f * c5 + 6.0f * c6)));
+  const df gdm = mul(u2, bracket(2.0f, 10.0f * d5 + 12.0f * d6, 0.0f));
+  const float gf = U * fmaf(0.25f, P, -1.0f / 6.0f);
+  df gm = mk(0.0f, 0.0f);
+  if (wide) gm = mul(mul(u, mk(0.16666667f, -4.967054e-09f)), bracket(1.5f, 6.0f * (d5 + d6), 0.0f));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    dv[c] = add_u(mul(fd, xx[c]), mul(gdm, hv[c]));
+    df hp = hv[c];
+    if (wide) hp = add_u(hp, mul(gm, hv[c]));
+    else hp.l = __fmaf_rn(gf, hv[c].h, hp.l);
+    dx[c] = add_u(hp, mul(fm1, xx[c]));
+  }
+  o.P = P;
+  o.Q = Q;
+  o.U = U;
+  return o;
+}
+
 // the same by the series to order 6, each sub-step as nq equal ones (h here is the sub-step over nq)
 __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int end, int M, int nq, bool wide) {
   const float fM = (float)M, fq = 1.0f / (float)nq;
@@ -178,9 +245,6 @@ __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int en
   float ri2s, ph, qh, uh;
 #pragma unroll 1
   for (int i = cj * nq, ni = end * nq; i < ni; ++i) {
-    // the series to order 6: its coefficients over u h^2 (drift_series()) are FP32 where what they
-    // multiply is below 1e-12: their error, unlike a rounding of x or v, is the same from one
-    // sub-step to the next and adds up.  With s > 1e-8 (wide) that leaves out c4 in f' and g - h.
     df xx[3], m[3], hv[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -188,53 +252,18 @@ __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int en
       m[c] = add_u(hn[c], mul(hk, d[c]));
       hv[c] = add(hv0[c], m[c]);
     }
-    const df_root q = root_fine(norm2(xx));
-    const df ri2 = inverse(q);
-    r3s = inverse_cube(q);
-    ri2s = ri2.h;
-    const df u = renorm(mul(mhh, r3s));                        // u h^2
-    const df pd = renorm(mul(dot3(xx, hv), ri2));              // p h
-    const float U = u.h, P = pd.h, P2 = P * P;
-    float Q;                                                   // q h^2
-    df c4d;                                                    // 4 c4 / (u h^2)
-    if (wide) {
-      const df qd = add(mul(norm2(hv), ri2), neg(u));
-      Q = qd.h;
-      c4d = mul(add(add(mul(qd, 3.0f), u), mul(sqr(pd), -15.0f)), mk(0.16666667f, -4.967054e-09f));
-    } else {
-      Q = fmaf(fmaf(hv[2].h, hv[2].h, fmaf(hv[1].h, hv[1].h, hv[0].h * hv[0].h)), ri2.h, -U);
-      c4d = mk((3.0f * Q - 15.0f * P2 + U) * (1.0f / 6.0f), 0.0f);
-    }
-    const float c4 = 0.25f * c4d.h;
-    const float c5 = P * (7.0f * P2 - 3.0f * Q - U) * 0.125f;
-    const float c6 = (P2 * (-945.0f * P2 + 630.0f * Q + 210.0f * U) - 45.0f * Q * Q - 24.0f * U * Q - U * U) *
-                     (1.0f / 720.0f);
-    const float d5 = (9.0f * Q - 45.0f * P2 + U) * (1.0f / 120.0f);
-    const float d6 = P * (14.0f * P2 - 6.0f * Q - U) * (1.0f / 24.0f);
-    // f - 1 = (u h^2/2) (-1 + p h + ...), h f' = u h^2 (-1 + 3/2 p h + ...), g' - 1 = (u h^2/2)
-    // (-1 + 2 p h + ...), g - h = h (u h^2/6) (-1 + 3/2 p h + ...)
-    auto bracket = [&](float k, float rest, float rest_l) {
-      const df p = mul(pd, k), t = fast_two_sum(-1.0f, p.h), b = fast_two_sum(t.h, rest);
-      return mk(b.h, __fadd_rn(__fadd_rn(b.l, t.l), __fadd_rn(p.l, rest_l)));
-    };
-    const df u2 = mk(0.5f * u.h, 0.5f * u.l);
-    const df fm1 = mul(u2, bracket(1.0f, 2.0f * (c4 + c5 + c6), 0.0f));
-    const df fd = mul(u, bracket(1.5f, c4d.h, c4d.l + (5.0f * c5 + 6.0f * c6)));
-    const df gdm = mul(u2, bracket(2.0f, 10.0f * d5 + 12.0f * d6, 0.0f));
-    const float gf = U * fmaf(0.25f, P, -1.0f / 6.0f);
-    df gm = mk(0.0f, 0.0f);
-    if (wide) gm = mul(mul(u, mk(0.16666667f, -4.967054e-09f)), bracket(1.5f, 6.0f * (d5 + d6), 0.0f));
+    df dx[3], dv[3];
+    const Series o = series_increments(xx, hv, mhh, wide, dx, dv);
+    r3s = o.r3s;
+    ri2s = o.ri2s;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      hn[c] = add(m[c], add_u(mul(fd, xx[c]), mul(gdm, hv[c])));
-      df hp = hv[c];
-      if (wide) hp = add_u(hp, mul(gm, hv[c]));
-      else hp.l = __fmaf_rn(gf, hv[c].h, hp.l);
-      dl[c] = add(dl[c], add_u(hp, mul(fm1, xx[c])));
+      hn[c] = add(m[c], dv[c]);
+      dl[c] = add(dl[c], dx[c]);
     }
-    ph = P;
-    qh = Q;
-    uh = U;
+    ph = o.P;
+    qh = o.Q;
+    uh = o.U;
     if ((i + 1) & (nq - 1)) {                                  // more of this sub-step to come
       hk = mk(0.0f, 0.0f);
       continue;
@@ -268,12 +297,13 @@ static __device__ __noinline__ int kepler_anchors(PairTab *T, int odd, double mu
 }
 
 // Runs the sub-steps of levels >= k with F_{k-1} = {q}, from the opening of a sub-step at level
-// k.  x, v: this lane's body (even lanes a, odd lanes b).  Returns 0 when level k has finished (k is
+// k.  x, v: this lane's body (even lanes a, odd lanes b); G, ea, eb: the group's table and units.  Returns 0 when level k has finished (k is
 // then k - 1), 1 when the pair may be in contact at the next check, or the scaled state does not
 // fit (k is that check's level; the general path takes the sub-step), 2 when the sub-step budget
 // ran out.
 __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lane, double *hs, int *cs,
-                                        PairTab *T, double (&x)[3], double (&v)[3], double gA, double gB,
+                                        PairTab *T, const GroupTab *G, int ea, int eb, double (&x)[3],
+                                        double (&v)[3], double gA, double gB,
                                         double pR0sq, double piR0, double pRcut, int &kio, int &plev_io,
                                         long long &substeps_io, int &deepest_io) {
   const int odd = lane & 1;
@@ -281,44 +311,24 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
   const int M = C.M, max_depth = C.max_depth, k0 = kio;
   const long long max_sub = C.max_substeps;
 
-  // scales: |x| < 2^(ea + 1), |v| < 2^(eb + 1) over both bodies
-  int ea, eb;
-  {
-    unsigned mx = 0u, mv = 0u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      mx = max(mx, (unsigned)__double2hiint(x[c]) & 0x7FFFFFFFu);
-      mv = max(mv, (unsigned)__double2hiint(v[c]) & 0x7FFFFFFFu);
-    }
-    ea = (int)(__reduce_max_sync(FULL, mx) >> 20) - 1023;
-    eb = (int)(__reduce_max_sync(FULL, mv) >> 20) - 1023;
-    // a state at rest takes the circular speed's scale
-    if (eb < -900) eb = ((((__double2hiint(C.mu) >> 20) & 0x7FF) - 1023) - ea) / 2;
-  }
   const int et = -2 * ea - eb;                          // scale of G m h
-  for (int L = lane; L < SYM_MAX_LEVELS + 2; L += 32) {
-    const double h = dp->hk[L], hh = 0.5 * h;
-    const df th = split(scale2(h, eb - ea)), ti = split(scale2(1.0 / h, ea - eb)), tm = split(scale2(C.mu * h * h, et + eb - ea));
-    const df ta = split(scale2(gB * hh, et)), tb = split(scale2(gA * hh, et));
-    const df tc = split(scale2(gB * hh * h, et + eb - ea)), td = split(scale2(gA * hh * h, et + eb - ea));
-    const df tr = split(scale2(pR0sq * dp->ck2[L], -2 * ea));
-    const int Ln = min(L + 1, SYM_MAX_LEVELS + 1);
-    const df tA = split(scale2(2.0 * piR0 * dp->invdc[L], ea)), tB = split(fma(-2.0 * dp->ck[Ln], dp->invdc[L], -1.0));
-    T->h[L] = make_float2(th.h, th.l);
-    T->mh[L] = make_float2(tm.h, tm.l);
+  // (a short visit is mostly this: entries of one pair only, and no level above k0 - 1)
+  for (int L = k0 - 1 + lane; L < SYM_MAX_LEVELS + 2; L += 32) {
+    const double h = dp->hk[L], hh = 0.5 * h, fa = gB * hh, fb = gA * hh;
+    const df ta = split(scale2(fa, et)), tb = split(scale2(fb, et));
+    const df tc = split(scale2(fa * h, et + eb - ea)), td = split(scale2(fb * h, et + eb - ea));
+    const df tr = split(scale2(pR0sq * dp->ck2[L], -2 * ea)), tA = split(scale2(2.0 * piR0 * dp->invdc[L], ea));
     T->ga[L] = make_float2(ta.h, ta.l);
     T->gb[L] = make_float2(tb.h, tb.l);
     T->ha[L] = make_float2(tc.h, tc.l);
     T->hb[L] = make_float2(td.h, td.l);
     T->R2[L] = make_float2(tr.h, tr.l);
     T->A[L] = make_float2(tA.h, tA.l);
-    T->B[L] = make_float2(tB.h, tB.l);
-    T->rh[L] = make_float2(ti.h, ti.l);
   }
   __syncwarp();
   {
     // the scaled quantities that must be normal FP32 numbers, with room for their products
-    const float hm = fabsf(T->h[k0].x), mm = fabsf(T->mh[k0].x), rr = T->R2[k0].x;
+    const float hm = fabsf(G->h[k0].x), mm = fabsf(G->mh[k0].x), rr = T->R2[k0].x;
     const bool fits = hm > 1e-18f && hm < 1e12f && mm > 1e-28f && mm < 1e12f && rr > 1e-24f && rr < 1e12f &&
                       fabsf(T->ga[k0].x) < 1e12f && fabsf(T->gb[k0].x) < 1e12f && abs(ea) < 400 && abs(eb) < 400;
     if (!fits) return 1;
@@ -347,9 +357,9 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
   df Ap, Bp;                               // of zone j - 1
   float hf, Rj, Rp, kmax;
   auto set_level = [&]() {
-    h = ld(T->h[j]); mh = ld(T->mh[j]); gg = ld(odd ? T->gb[j] : T->ga[j]);
+    h = ld(G->h[j]); mh = ld(G->mh[j]); gg = ld(odd ? T->gb[j] : T->ga[j]);
     R2p = ld(T->R2[j - 1]); R2j = ld(T->R2[j]); R2n = ld(T->R2[j + 1]);
-    Ap = ld(T->A[j - 1]); Bp = ld(T->B[j - 1]);
+    Ap = ld(T->A[j - 1]); Bp = ld(G->B[j - 1]);
     hf = h.h;
     Rj = R2j.h > 0.0f ? R2j.h * rsqrt_seed(R2j.h) * 1.000001f : 0.0f;   // not below R_j
     Rp = R2p.h > 0.0f ? R2p.h * rsqrt_seed(R2p.h) * 0.999999f : 0.0f;   // not above R_{j-1}
@@ -451,7 +461,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
         const bool zero = r2.h < R2n.h || !(r2.h < R2p.h);     // w_j = 0 outside [R_{j+1}, R_{j-1})
         const int z = fl ? j : j - 1;
         if (zc != z && !zero) {
-          yp = zone_odd(r, ld(T->A[z]), ld(T->B[z]));
+          yp = zone_odd(r, ld(T->A[z]), ld(G->B[z]));
           zc = z;
         }
         // w_j = g_j inside R_j, 1 - g_{j-1} outside
@@ -627,7 +637,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
         cj = 0;
         substeps += up + M;                                // the levels below, and the M of level j
       }
-      const df rh = mul(ld(T->rh[j]), (float)nq);
+      const df rh = mul(ld(G->rh[j]), (float)nq);
 #pragma unroll
       for (int c = 0; c < 3; ++c) { nu[c] = renorm(mul(rh, S.hn[c])); dl[c] = S.dl[c]; d[c] = S.d[c]; }
       r3s = S.r3s; ri2s = S.ri2s; r2 = S.r2; r = S.r; r3 = S.r3; yp = S.yp;
