@@ -300,25 +300,18 @@ __device__ __forceinline__ bool small_levels(const Dev &D, const GroupCtx &C, co
       __syncwarp();
       return;
     }
-    const bool wide = so >= 1e-8f;
-    const int nq = so <= 2.0e-6f ? 1 : (so <= 8.0e-6f ? 4 : (so <= 3.2e-5f ? 8 : 16));   // s <= 5e-7 each
-    const float fq = 1.0f / (float)nq, fn = (float)nq;
-    const df hq = mk(fq * h.h, fq * h.l), mq = mk(fq * fq * mh.h, fq * fq * mh.l), iq = mk(fn * ih.h, fn * ih.l);
     if (go) {
-#pragma unroll 1
-      for (int i = 0; i < nq; ++i) {
-        df xx[3], hv[3], dx[3], dv[3];
+      df xx[3], hv[3], dx[3], dv[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          xx[c] = add(x0[c], dl[c]);
-          hv[c] = mul(hq, add(v0[c], nu[c]));
-        }
-        series_increments(xx, hv, mq, wide, dx, dv);
+      for (int c = 0; c < 3; ++c) {
+        xx[c] = add(x0[c], dl[c]);
+        hv[c] = mul(h, add(v0[c], nu[c]));
+      }
+      series_increments(xx, hv, mh, so >= 1e-8f, so > 2.0e-6f, dx, dv);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          dl[c] = add(dl[c], dx[c]);
-          nu[c] = add(nu[c], mul(iq, dv[c]));
-        }
+      for (int c = 0; c < 3; ++c) {
+        dl[c] = add(dl[c], dx[c]);
+        nu[c] = add(nu[c], mul(ih, dv[c]));
       }
     }
     __syncwarp();

@@ -36,8 +36,8 @@
 //     x' = x + h v - (u h^2/2) x,  v' = v - u h (1 - 3/2 p h) (x + h/2 v); 1/r^3 of the sun distance
 //     is carried along by the factor (1 + w)^(-3/2), w = 2 p h + q h^2 the relative change of r^2
 //     (|w| < 2e-6, formed in FP32 to 2^-43), and formed in full at every anchor;
-//   s <= 1.3e-4: the Lagrange f and g series of drift_series() to order 6, 1/r^3, u, p and the leading
-//     coefficients in double-float; sub-steps with s > 2e-6 as 4 to 16 equal drifts;
+//   s <= 1.3e-4: the Lagrange f and g series, to order 6 as in drift_series() and above s = 2e-6 to
+//     order 10, 1/r^3, u, p and the leading coefficients in double-float;
 //   longer intervals: the FP64 Kepler solver on the anchors.
 //
 // Cost and bound (one GB300 at 2.07 GHz).  A cleared order-2 sub-step is ~410 warp instructions, 95 %
@@ -169,54 +169,115 @@ __device__ __forceinline__ void run_order2(Run &S, df gh, df mhh, int cj, int en
   S.ph = ph; S.qh = qh; S.uh = uh;
 }
 
-// The Lagrange f and g series of drift_series() to order 6 at position xx with velocity hv / h: increments
-// dx of the position and dv / h of the velocity.  mhh: mu h^2.
+// The Lagrange f and g series at position xx with velocity hv / h: increments dx of the position and
+// dv / h of the velocity.  mhh: mu h^2.  Orders to 6 as in drift_series(), and to 10 for intervals with
+// s > 2e-6 (far).
 struct Series {
   df r3s;                          // 1/r^3 from the sun
   float ri2s, P, Q, U;             // 1/r^2, p h, q h^2, u h^2
 };
-__device__ __forceinline__ Series series_increments(const df (&xx)[3], const df (&hv)[3], df mhh, bool wide,
+// Without the orders above 6 such an interval was 4 to 16 equal drifts: a level of them 2.24 -> 1.32 us
+// per sub-step, with the levels around it; 260 disks of 500 to 4,000 bodies 3 % faster (geometric mean).
+// Orders 7 to 10 of both series over U = u h^2, from the recurrences of u' = -3 u p, p' = q - 2 p^2,
+// w' = -2 p (u + w), w = v^2/r^2 = q + u, f'' = -u f: sums of c_k, k c_k, g_k and k g_k.
+// (Called, not inlined: its 40 temporaries would be taken from the sub-steps that do not need it.)
+static __device__ __noinline__ float4 series_tail(float U, float P, float W) {
+  float e[9], p[8], w[8], c[11], g[11];
+  e[0] = 1.0f;
+  p[0] = P;
+  w[0] = W;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    float a = 0.0f, b = 0.0f, m = 0.0f;
+#pragma unroll
+    for (int j = 0; j <= k; ++j) {
+      a = fmaf(e[j], p[k - j], a);
+      b = fmaf(p[j], p[k - j], b);
+      m = fmaf(p[j], fmaf(U, e[k - j], w[k - j]), m);
+    }
+    const float i = 1.0f / (float)(k + 1);
+    e[k + 1] = -3.0f * i * a;
+    if (k < 7) {
+      p[k + 1] = i * (fmaf(-U, e[k], w[k]) - 2.0f * b);
+      w[k + 1] = -2.0f * i * m;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k <= 8; ++k) {                               // c_2 .. c_10, g_3 .. g_10
+    float a = 0.0f, b = 0.0f;
+#pragma unroll
+    for (int j = 0; j + 2 <= k; ++j) {
+      a = fmaf(e[j], c[k - j], a);
+      if (j + 3 <= k) b = fmaf(e[j], g[k - j], b);
+    }
+    const float i = -1.0f / (float)((k + 1) * (k + 2));
+    c[k + 2] = i * fmaf(U, a, e[k]);
+    if (k > 0) g[k + 2] = i * fmaf(U, b, e[k - 1]);
+  }
+  return make_float4((c[7] + c[8]) + (c[9] + c[10]),
+                     fmaf(7.0f, c[7], 8.0f * c[8]) + fmaf(9.0f, c[9], 10.0f * c[10]),
+                     (g[7] + g[8]) + (g[9] + g[10]),
+                     fmaf(7.0f, g[7], 8.0f * g[8]) + fmaf(9.0f, g[9], 10.0f * g[10]));
+}
+__device__ __forceinline__ Series series_increments(const df (&xx)[3], const df (&hv)[3], df mhh, bool wide, bool far,
                                                     df (&dx)[3], df (&dv)[3]) {
-  // its coefficients over u h^2 (drift_series()) are FP32 where what they multiply is below 1e-12:
-  // their error, unlike a rounding of x or v, is the same from one sub-step to the next and adds up.
-  // With s > 1e-8 (wide) that leaves out c4 in f' and g - h.
+  // Coefficients over u h^2: FP32 where what they multiply is below 1e-17 of x and 1e-16 of v: their error,
+  // unlike a rounding of x or v, is the same from one sub-step to the next and adds up.  With
+  // s > 1e-8 (wide) that leaves out c4 in f' and g - h, with s > 2e-6 c4 everywhere, c5 in f' and the
+  // fifth order of g' too.
   Series o;
+  const df sixth = mk(0.16666667f, -4.967054e-09f);
   const df_root q = root_fine(norm2(xx));
   const df ri2 = inverse(q);
   o.r3s = inverse_cube(q);
   o.ri2s = ri2.h;
-  const df u = renorm(mul(mhh, o.r3s));                        // u h^2
+  const df u = renorm(mul(mhh, o.r3s));                      // u h^2
   const df pd = renorm(mul(dot3(xx, hv), ri2));              // p h
   const float U = u.h, P = pd.h, P2 = P * P;
   float Q;                                                   // q h^2
-  df c4d;                                                    // 4 c4 / (u h^2)
+  df qd, c4d;                                                // 4 c4
   if (wide) {
-    const df qd = add(mul(norm2(hv), ri2), neg(u));
+    qd = add(mul(norm2(hv), ri2), neg(u));
     Q = qd.h;
-    c4d = mul(add(add(mul(qd, 3.0f), u), mul(sqr(pd), -15.0f)), mk(0.16666667f, -4.967054e-09f));
+    c4d = mul(add(add(mul(qd, 3.0f), u), mul(sqr(pd), -15.0f)), sixth);
   } else {
     Q = fmaf(fmaf(hv[2].h, hv[2].h, fmaf(hv[1].h, hv[1].h, hv[0].h * hv[0].h)), ri2.h, -U);
+    qd = mk(Q, 0.0f);
     c4d = mk((3.0f * Q - 15.0f * P2 + U) * (1.0f / 6.0f), 0.0f);
   }
-  const float c4 = 0.25f * c4d.h;
   const float c5 = P * (7.0f * P2 - 3.0f * Q - U) * 0.125f;
   const float c6 = (P2 * (-945.0f * P2 + 630.0f * Q + 210.0f * U) - 45.0f * Q * Q - 24.0f * U * Q - U * U) *
                    (1.0f / 720.0f);
   const float d5 = (9.0f * Q - 45.0f * P2 + U) * (1.0f / 120.0f);
   const float d6 = P * (14.0f * P2 - 6.0f * Q - U) * (1.0f / 24.0f);
+  // the brackets' terms from order 4 (5 in g) on
+  df fr = mk(0.5f * c4d.h + 2.0f * (c5 + c6), 0.0f), fdr = mk(c4d.h, c4d.l + (5.0f * c5 + 6.0f * c6));
+  df gr = mk(10.0f * d5 + 12.0f * d6, 0.0f);
+  float gmr = 6.0f * (d5 + d6);
+  if (far) {
+    const float4 t = series_tail(U, P, Q + U);
+    // 5 c5 = 5/8 P (7 P^2 - 3 Q - U), 10 d5 = 3/2 (4 c4) - U / 6
+    const df c5d = mul(mul(pd, 0.625f), add(add(mul(sqr(pd), 7.0f), mul(qd, -3.0f)), neg(u)));
+    fr = mk(0.5f * c4d.h, 0.5f * c4d.l + 2.0f * (c5 + c6 + t.x));
+    fdr = add(c4d, c5d);
+    fdr.l += 6.0f * c6 + t.y;
+    gr = add(mk(1.5f * c4d.h, 1.5f * c4d.l), neg(mul(u, sixth)));
+    gr.l += 12.0f * d6 + 2.0f * t.w;
+    gmr += 6.0f * t.z;
+  }
   // f - 1 = (u h^2/2) (-1 + p h + ...), h f' = u h^2 (-1 + 3/2 p h + ...), g' - 1 = (u h^2/2)
   // (-1 + 2 p h + ...), g - h = h (u h^2/6) (-1 + 3/2 p h + ...)
-  auto bracket = [&](float k, float rest, float rest_l) {
-    const df p = mul(pd, k), t = fast_two_sum(-1.0f, p.h), b = fast_two_sum(t.h, rest);
-    return mk(b.h, __fadd_rn(__fadd_rn(b.l, t.l), __fadd_rn(p.l, rest_l)));
+  auto bracket = [&](float k, df rest) {
+    const df p = mul(pd, k), t = fast_two_sum(-1.0f, p.h), b = fast_two_sum(t.h, rest.h);
+    return mk(b.h, __fadd_rn(__fadd_rn(b.l, t.l), __fadd_rn(p.l, rest.l)));
   };
   const df u2 = mk(0.5f * u.h, 0.5f * u.l);
-  const df fm1 = mul(u2, bracket(1.0f, 2.0f * (c4 + c5 + c6), 0.0f));
-  const df fd = mul(u, bracket(1.5f, c4d.h, c4d.l + (5.0f * c5 + 6.0f * c6)));
-  const df gdm = mul(u2, bracket(2.0f, 10.0f * d5 + 12.0f * d6, 0.0f));
+  const df fm1 = mul(u2, bracket(1.0f, fr));
+  const df fd = mul(u, bracket(1.5f, fdr));
+  const df gdm = mul(u2, bracket(2.0f, gr));
   const float gf = U * fmaf(0.25f, P, -1.0f / 6.0f);
   df gm = mk(0.0f, 0.0f);
-  if (wide) gm = mul(mul(u, mk(0.16666667f, -4.967054e-09f)), bracket(1.5f, 6.0f * (d5 + d6), 0.0f));
+  if (wide) gm = mul(mul(u, sixth), bracket(1.5f, mk(gmr, 0.0f)));
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     dv[c] = add_u(mul(fd, xx[c]), mul(gdm, hv[c]));
@@ -231,20 +292,20 @@ __device__ __forceinline__ Series series_increments(const df (&xx)[3], const df 
   return o;
 }
 
-// the same by the series to order 6, each sub-step as nq equal ones (h here is the sub-step over nq)
-__device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int end, int M, int nq, bool wide) {
-  const float fM = (float)M, fq = 1.0f / (float)nq;
+// the same by the series
+__device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int end, int M, bool wide, bool far) {
+  const float fM = (float)M;
   df x0[3], d0[3], hv0[3], hn[3], dl[3], d[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    x0[c] = S.x0[c]; d0[c] = S.d0[c]; hv0[c] = mk(fq * S.hv0[c].h, fq * S.hv0[c].l);
+    x0[c] = S.x0[c]; d0[c] = S.d0[c]; hv0[c] = S.hv0[c];
     hn[c] = S.hn[c]; dl[c] = S.dl[c]; d[c] = S.d[c];
   }
   const df Ap = S.Ap, Bp = S.Bp;
   df hk = S.hk, r3s, r2, r, r3, yp;
   float ri2s, ph, qh, uh;
 #pragma unroll 1
-  for (int i = cj * nq, ni = end * nq; i < ni; ++i) {
+  for (int i = cj; i < end; ++i) {
     df xx[3], m[3], hv[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -253,7 +314,7 @@ __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int en
       hv[c] = add(hv0[c], m[c]);
     }
     df dx[3], dv[3];
-    const Series o = series_increments(xx, hv, mhh, wide, dx, dv);
+    const Series o = series_increments(xx, hv, mhh, wide, far, dx, dv);
     r3s = o.r3s;
     ri2s = o.ri2s;
 #pragma unroll
@@ -264,17 +325,13 @@ __device__ __forceinline__ void run_series(Run &S, df gh, df mhh, int cj, int en
     ph = o.P;
     qh = o.Q;
     uh = o.U;
-    if ((i + 1) & (nq - 1)) {                                  // more of this sub-step to come
-      hk = mk(0.0f, 0.0f);
-      continue;
-    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const float oh = __shfl_xor_sync(FULL, dl[c].h, 1), ol = __shfl_xor_sync(FULL, dl[c].l, 1);
       const df t = two_sum(oh, -dl[c].h), e = two_sum(d0[c].h, t.h);
       d[c] = fast_two_sum(e.h, __fadd_rn(e.l, __fadd_rn(t.l, __fadd_rn(__fsub_rn(ol, dl[c].l), d0[c].l))));
     }
-    RUN_KICK(i + 1 == M * nq ? fM : 0.0f);
+    RUN_KICK(i + 1 == M ? fM : 0.0f);
   }
 
 #pragma unroll
@@ -578,9 +635,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
       // longer, weight g.  One test clears the next M sub-steps at once: in them |d| cannot change by more
       // than M times h |dv| and what the kicks and the sun's tide can add to it; the sub-steps themselves
       // then have no decision left.  Without that clearance the run is this one sub-step.
-      // Velocities and kicks here are times h / nq: a sub-step too long for the series (s > 2e-6) is taken
-      // as nq = 4 to 16 equal ones of s <= 5e-7 without a kick between them, which is the same motion (the
-      // series' first omitted term, 1e-17 at s = 2e-6, is then added up 16 times).
+      // Velocities and kicks in a run are times h.
       const float fM = (float)M;
       auto clear = [&](float speed, float u) {             // speed: h |dv| here; u: u h^2
         const float need = fM * (speed + fM * (kmax + 4.0f * fabsf(u) * Rp)) * 1.0001f;
@@ -590,24 +645,19 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
       int end = run ? M : cj + 1;
       substeps += end - 1 - cj;                            // (this one is counted)
       if (order2 && !fresh) sun();
-      const bool wide = so >= 1e-8f;
-      const int nq = so <= 2.0e-6f ? 1 : (so <= 8.0e-6f ? 4 : (so <= 3.2e-5f ? 8 : 16));   // s <= 5e-7 each
-      const float fq = 1.0f / (float)nq;                   // a power of two: every scaling by it is exact
-      const df hq = mk(fq * h.h, fq * h.l);
-      const df g2 = ld(odd ? T->hb[j] : T->ha[j]);
-      const df gh = mk(fq * g2.h, fq * g2.l);              // G m h hq / 2
-      const df mhh = mk(fq * fq * mh.h, fq * fq * mh.l);   // mu hq^2
+      const bool wide = so >= 1e-8f, beyond = so > 2.0e-6f;
+      const df gh = ld(odd ? T->hb[j] : T->ha[j]);           // G m h^2 / 2
       Run S;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         S.x0[c] = x0[c]; S.d0[c] = d0[c]; S.hv0[c] = hv0[c];
-        S.hn[c] = renorm(mul(hq, nu[c])); S.dl[c] = dl[c]; S.d[c] = d[c];
+        S.hn[c] = renorm(mul(h, nu[c])); S.dl[c] = dl[c]; S.d[c] = d[c];
       }
-      S.hk = mul(hc, hq);
+      S.hk = mul(hc, h);
       S.Ap = Ap; S.Bp = Bp; S.r3s = r3s; S.ri2s = ri2s;
       for (;;) {
-        if (order2) run_order2(S, gh, mhh, cj, end, M);
-        else run_series(S, gh, mhh, cj, end, M, nq, wide);
+        if (order2) run_order2(S, gh, mh, cj, end, M);
+        else run_series(S, gh, mh, cj, end, M, wide, beyond);
         t_el = fmaf((float)(end - cj), fabsf(hf), t_el);
         n_el += end - cj;
         cj = end - 1;
@@ -617,18 +667,18 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
         if (j - up < k0 || n_el > ANCHOR_N || t_el > (order2 ? 0.03125f * t_lim : t_lim) || substeps + M + up >= max_sub)
           break;
         // h |dv| with the opening kick of level j (within kmax of what the test there sees)
-        float s2 = 0.0f, sa = vsum * fabsf(hq.h);
+        float s2 = 0.0f, sa = vsum * fabsf(hf);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const float uf = fmaf(S.hk.h, S.d[c].h, S.hn[c].h), uo = __shfl_xor_sync(FULL, uf, 1);
-          const float du = fmaf(hq.h, dv0[c], uo - uf);
+          const float du = fmaf(hf, dv0[c], uo - uf);
           s2 = fmaf(du, du, s2);
           sa += fabsf(uo) + fabsf(uf);
         }
         r = S.r;
         const float so1 = fmaxf(fmaxf(fabsf(S.uh), S.ph * S.ph), fabsf(S.qh));
-        const float fn = (float)nq, hdv1 = fn * (s2 * rsqrt_seed(fmaxf(s2, 1e-36f)) * 1.0001f + sa * 2.3841858e-7f);
-        if (!__all_sync(FULL, clear(hdv1, fn * fn * S.uh) && so1 < (order2 ? 5e-13f : (wide ? 2.0e-6f : 1e-8f)))) break;
+        const float hdv1 = s2 * rsqrt_seed(fmaxf(s2, 1e-36f)) * 1.0001f + sa * 2.3841858e-7f;
+        if (!__all_sync(FULL, clear(hdv1, S.uh) && so1 < (order2 ? 5e-13f : (beyond ? 1.28e-4f : (wide ? 2.0e-6f : 1e-8f))))) break;
         const int t = cs[j - up] + 1;
         __syncwarp();
         for (int i = 1; i < up; ++i) cs[j - i] = 0;
@@ -637,7 +687,7 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
         cj = 0;
         substeps += up + M;                                // the levels below, and the M of level j
       }
-      const df rh = mul(ld(G->rh[j]), (float)nq);
+      const df rh = ld(G->rh[j]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) { nu[c] = renorm(mul(rh, S.hn[c])); dl[c] = S.dl[c]; d[c] = S.d[c]; }
       r3s = S.r3s; ri2s = S.ri2s; r2 = S.r2; r = S.r; r3 = S.r3; yp = S.yp;

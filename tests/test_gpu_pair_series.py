@@ -96,3 +96,12 @@ def test_pair_variants(orc, sy, what):
     if what == "SI_units":
         x, v, m, kw = x * AU, v * AU / YR, m * MSUN, dict(dt=0.05 * YR, G=6.6743e-11, m0=MSUN)
     _check(orc, sy, x, v, m, np.full(2, 1e-9 * (AU if what == "SI_units" else 1.0)), kw)
+
+
+@pytest.mark.parametrize("a,e,dt", [(7.4, 0.0, 0.11), (5.0, 0.0, 0.133), (5.0, 0.0, 0.135), (6.0, 0.6, 0.05), (9.0, 0.3, 0.5)])
+def test_series_to_order_10(orc, sy, a, e, dt):
+    """Levels on both sides of s = 2e-6 (order 6 to 10) and of s = 1.28e-4 (order 10 to the Kepler
+    solver), near pericentre of eccentric orbits too: a wide pair that stays on shallow levels."""
+    m = np.array([3e-8, 2e-8])
+    x, v = _pair(a, e, 0.02, 6e-3 * a, 0.1, m)
+    _check(orc, sy, x, v, m, np.full(2, 1e-9), dict(dt=dt))
