@@ -703,7 +703,7 @@ def run_ours(args):
                         if ne == args.steps else f"the first {ne} of the timed steps'"},
                 # per timed step: the step's 12 kernels plus the per-call statistics reset (the
                 # loop times each step as its own call; the launch list shows the same 13)
-                "gpu_launches": args.steps * 13,
+                "gpu_launches": args.steps * 12,
                 "clocks": clk, "wall_s": wall, "second": second, "rates": rates,
                 "chain_vs_cpu": chain, "batched": batched, "served": served, "field": field}
         print(json.dumps(line), flush=True)

@@ -91,6 +91,7 @@ struct symba_pool {
   long long mcap = 0, macros_used = 0;       // macro-tiles: capacity and in use
   long long npart_hwm = 0;
   int ndisks = 0;
+  int n_max = 0;                // bodies of the largest system
   std::vector<void *> allocs;
   unsigned long long *eacc = nullptr;
   double *eout = nullptr;
@@ -176,6 +177,7 @@ int rebuild(symba_pool *P) {
   std::vector<DiskDesc> descs(P->max_disks);
   std::vector<int2> fblk;
   bool any_discard = false;
+  int n_max = 0;
   for (int d = 0; d < P->max_disks; ++d) {
     Slot &s = P->slots[d];
     DiskDesc &dd = descs[d];
@@ -183,6 +185,7 @@ int rebuild(symba_pool *P) {
     if (!s.active) continue;
     dd.off = s.off; dd.n = s.n; dd.nm = s.nm; dd.nb = s.nb; dd.nbm = s.nbm;
     dd.tile_base = (int)tiles.size();
+    n_max = std::max(n_max, s.n);
     dd.ntiles = s.nmacro;
     dd.pair_base = s.pair_base; dd.pair_cap = s.pair_cap;
     dd.group_base = s.off / 2;
@@ -201,6 +204,7 @@ int rebuild(symba_pool *P) {
     for (int B = s.nbm; B < s.nb; ++B) fblk.push_back(make_int2(d, b0 + B));
   }
   P->ndisks = hw;
+  P->n_max = n_max;
   P->npart_hwm = phw;
   P->any_discard = any_discard;
   P->D.ndisks = hw;
@@ -234,8 +238,7 @@ int rebuild(symba_pool *P) {
 void enqueue_step(symba_pool *P, cudaEvent_t rec0 = nullptr, cudaEvent_t rec1 = nullptr) {
   const Dev &D = P->D;
   const long long np = P->npart_hwm;
-  launch_prologue(D, P->ndisks, P->stream);
-  launch_sundrift(D, np, 1, P->stream);
+  launch_open(D, np, P->ndisks, P->stream);
   launch_trap(D, P->L, 1, P->precision, P->stream);
   launch_field(D, 1, P->precision, P->stream);
   launch_reduce(D, np, P->precision, P->stream);
@@ -250,8 +253,7 @@ void enqueue_step(symba_pool *P, cudaEvent_t rec0 = nullptr, cudaEvent_t rec1 = 
   launch_field(D, 2, P->precision, P->stream);
   launch_reduce(D, np, P->precision, P->stream);
   if (P->any_discard) launch_discard(D, np, P->stream);
-  launch_momentum(D, P->ndisks, P->stream);
-  launch_sundrift(D, np, 0, P->stream);
+  launch_momentum(D, P->ndisks, np, P->n_max, true, P->stream);
 }
 
 __global__ void k_reset_call(DiskStat *st, int nd) {
@@ -277,8 +279,7 @@ int pool_profile(symba_pool *P, int nsteps, double *phase_ms) {
   int rc = SYMBA_OK;
   for (int step = 0; step < nsteps && rc == SYMBA_OK; ++step) {
     cudaEventRecord(ev[0], s);
-    launch_prologue(D, P->ndisks, s);
-    launch_sundrift(D, np, 1, s);
+    launch_open(D, np, P->ndisks, s);
     cudaEventRecord(ev[1], s);
     launch_trap(D, P->L, 1, P->precision, s);
     launch_field(D, 1, P->precision, s);
@@ -299,9 +300,8 @@ int pool_profile(symba_pool *P, int nsteps, double *phase_ms) {
     launch_reduce(D, np, P->precision, s);
     if (P->any_discard) launch_discard(D, np, s);
     cudaEventRecord(ev[8], s);
-    launch_momentum(D, P->ndisks, s);
-    cudaEventRecord(ev[9], s);
-    launch_sundrift(D, np, 0, s);
+    launch_momentum(D, P->ndisks, np, P->n_max, true, s);
+    cudaEventRecord(ev[9], s);             // (the closing drift is launched with the momentum)
     cudaEventRecord(ev[10], s);
     if (cudaEventSynchronize(ev[10]) != cudaSuccess) { rc = SYMBA_E_CUDA; break; }
     for (int k = 0; k < SYMBA_NPHASES; ++k) {
@@ -465,7 +465,7 @@ int pool_admit(symba_pool *P, const symba_params *p, int n, int nm, const double
   if ((st = stage_in(sh, rhill, sizeof(double) * n, P->stream)) != SYMBA_OK) return st;
   launch_init_state(P->D, d, n, (const double *)sx.dev, (const double *)sv.dev, (const double *)sm.dev,
                     (const double *)sr.dev, (const double *)sh.dev, rhill == nullptr ? 1 : 0, P->stream);
-  launch_momentum(P->D, P->ndisks, P->stream);
+  launch_momentum(P->D, P->ndisks, P->npart_hwm, P->n_max, false, P->stream);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(P->stream));  // staging buffers are freed on return
   if (slot) *slot = d;
@@ -552,7 +552,7 @@ int set_state(symba_pool *P, int d, const double *x, const double *v) {
   if ((st = stage_in(sx, x, sizeof(double) * 3 * n, P->stream)) != SYMBA_OK) return st;
   if ((st = stage_in(sv, v, sizeof(double) * 3 * n, P->stream)) != SYMBA_OK) return st;
   launch_scatter_state(P->D, d, n, (const double *)sx.dev, (const double *)sv.dev, P->stream);
-  launch_momentum(P->D, P->ndisks, P->stream);
+  launch_momentum(P->D, P->ndisks, P->npart_hwm, P->n_max, false, P->stream);
   CK(cudaMemsetAsync(&P->D.stat[d].status, 0, sizeof(int), P->stream));
   CK(cudaGetLastError());
   if (sx.own || sv.own) CK(cudaStreamSynchronize(P->stream));

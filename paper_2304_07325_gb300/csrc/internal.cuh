@@ -302,32 +302,33 @@ __device__ inline void sa_carry(unsigned long long *dig) {
   }
 }
 
-__device__ inline double sa_round(const unsigned long long *in) {
+// (digits outside [lo, hi) are zero and stay zero; d[hi - 1] has room for the sign)
+__device__ inline double sa_round(const unsigned long long *in, int lo = 0, int hi = SA_NDIG) {
   if (in[SA_NDIG] != 0ull) return __longlong_as_double(0x7FF8000000000000ll);
   long long d[SA_NDIG];
-  for (int k = 0; k < SA_NDIG; ++k) d[k] = (long long)in[k];
-  for (int k = 0; k < SA_NDIG - 1; ++k) {
+  for (int k = lo; k < hi; ++k) d[k] = (long long)in[k];
+  for (int k = lo; k < hi - 1; ++k) {
     const long long c = d[k] >> 32;
     d[k] -= c * 4294967296ll;
     d[k + 1] += c;
   }
-  const bool neg = d[SA_NDIG - 1] < 0;
+  const bool neg = d[hi - 1] < 0;
   if (neg) {
-    for (int k = 0; k < SA_NDIG; ++k) d[k] = -d[k];
-    for (int k = 0; k < SA_NDIG - 1; ++k) {
+    for (int k = lo; k < hi; ++k) d[k] = -d[k];
+    for (int k = lo; k < hi - 1; ++k) {
       const long long c = d[k] >> 32;
       d[k] -= c * 4294967296ll;
       d[k + 1] += c;
     }
   }
-  int t = SA_NDIG - 1;
-  while (t >= 0 && d[t] == 0) --t;
-  if (t < 0) return 0.0;
+  int t = hi - 1;
+  while (t >= lo && d[t] == 0) --t;
+  if (t < lo) return 0.0;
   const unsigned long long dt = (unsigned long long)d[t];
-  const unsigned long long d1 = t >= 1 ? (unsigned long long)d[t - 1] : 0ull;
-  const unsigned long long d2 = t >= 2 ? (unsigned long long)d[t - 2] : 0ull;
+  const unsigned long long d1 = t >= lo + 1 ? (unsigned long long)d[t - 1] : 0ull;
+  const unsigned long long d2 = t >= lo + 2 ? (unsigned long long)d[t - 2] : 0ull;
   bool sticky = false;
-  for (int k = 0; k < t - 2; ++k) sticky |= (d[k] != 0);
+  for (int k = lo; k < t - 2; ++k) sticky |= (d[k] != 0);
   const int lz = __clz((unsigned)dt);
   const unsigned long long H = (dt << 32) | d1;
   unsigned long long T;
@@ -343,7 +344,7 @@ __device__ inline double sa_round(const unsigned long long *in) {
   if (E < -1022) {
     // below the normal range the exact sum (a multiple of 2^-1074) is representable
     r = 0.0;
-    for (int k = t; k >= 0; --k) r += ldexp((double)d[k], 32 * k - 1088);
+    for (int k = t; k >= lo; --k) r += ldexp((double)d[k], 32 * k - 1088);
   } else {
     unsigned long long mant = T >> 11;
     const bool rbit = (T >> 10) & 1ull;
@@ -356,6 +357,23 @@ __device__ inline double sa_round(const unsigned long long *in) {
     else r = ldexp((double)mant, E - 52);
   }
   return neg ? -r : r;
+}
+// the same by a warp (every lane calls it): the walk is one thread's, over the digits in use only -- a sum
+// of like terms uses 5 to 8 of the 68 -- and the digits are read by all lanes at once
+__device__ inline double sa_round_warp(const unsigned long long *in, int lane) {
+  static_assert(SA_NDIG <= 96, "three digits a lane");
+  int lo = SA_NDIG, hi = -1;
+#pragma unroll
+  for (int k = 2; k >= 0; --k) {
+    const unsigned m = __ballot_sync(0xffffffffu, 32 * k + lane < SA_NDIG && in[32 * k + lane] != 0ull);
+    if (m) {
+      lo = 32 * k + __ffs(m) - 1;
+      if (hi < 0) hi = 32 * k + 31 - __clz(m);
+    }
+  }
+  double r = 0.0;
+  if (lane == 0) r = hi < 0 ? sa_round(in, 0, 1) : sa_round(in, lo, min(hi + 3, SA_NDIG));
+  return __shfl_sync(0xffffffffu, r, 0);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -469,8 +487,10 @@ void launch_setup_disk(const Dev &D, int d, cudaStream_t s);
 void launch_init_state(const Dev &D, int d, int n, const double *xh, const double *vh,
                        const double *m, const double *rad, const double *rh, int compute_rh,
                        cudaStream_t s);
-void launch_momentum(const Dev &D, int ndisks, cudaStream_t s);
-void launch_sundrift(const Dev &D, long long npart, int pre, cudaStream_t s);
+// total momentum of every system (n_max: bodies of the largest); drift: and the closing sun drift
+void launch_momentum(const Dev &D, int ndisks, long long npart, int n_max, bool drift, cudaStream_t s);
+// opening sun drift of a step, with the reset of the per-step counters
+void launch_open(const Dev &D, long long npart, int ndisks, cudaStream_t s);
 void launch_trap(const Dev &D, const LaunchCfg &L, int mode, int precision, cudaStream_t s);
 void launch_reduce(const Dev &D, long long npart, int precision, cudaStream_t s);
 void launch_split(const Dev &D, long long npart, cudaStream_t s);
@@ -484,7 +504,6 @@ void launch_gather_state(const Dev &D, int d, int n, double *x, double *v, doubl
                          int *alive, double *rh, cudaStream_t s);
 void launch_scatter_state(const Dev &D, int d, int n, const double *x, const double *v,
                           cudaStream_t s);
-void launch_prologue(const Dev &D, int ndisks, cudaStream_t s);
 void launch_field(const Dev &D, int mode, int precision, cudaStream_t s);
 void launch_discard(const Dev &D, long long npart, cudaStream_t s);
 int trap_blocks_per_sm(int precision);

@@ -109,13 +109,17 @@ __global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const do
   gtop = __reduce_max_sync(0xffffffffu, gtop);
   if (lane == 0) { atomicMax(&top[0], xtop); atomicMax(&top[1], gtop); }
   __syncthreads();
+  __shared__ double sum[4];
+  if (threadIdx.x < 128) {
+    const double r = sa_round_warp(acc[threadIdx.x >> 5], lane);
+    if (lane == 0) sum[threadIdx.x >> 5] = r;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     D.disks[d].kex = (top[0] >> 20) - 1023;
     D.disks[d].keg = top[1] ? (top[1] >> 20) - 1023 : 0;
-    const DiskDesc dd = D.disks[d];
-    const double Mt = sa_round(acc[3]);
-    const double denom = __dadd_rn(dd.m0, Mt);
-    for (int c = 0; c < 3; ++c) q_out[c] = __ddiv_rn(sa_round(acc[c]), denom);
+    const double denom = __dadd_rn(D.disks[d].m0, sum[3]);
+    for (int c = 0; c < 3; ++c) q_out[c] = __ddiv_rn(sum[c], denom);
   }
 }
 
@@ -171,41 +175,26 @@ void launch_init_state(const Dev &D, int d, int n, const double *xh, const doubl
 }
 
 // --------------------------------------------------------------------------------------------
-// per-step prologue: reset the per-step counters
-// --------------------------------------------------------------------------------------------
-__global__ void k_prologue(Dev D, int ndisks) {
-  const int t = threadIdx.x;
-  if (t < 4) D.work[t] = 0;
-  if (t == 0) *D.rec_total = 0;
-  for (int d = t; d < ndisks; d += blockDim.x) {
-    D.stat[d].npairs = 0;
-    D.stat[d].ngroups = 0;
-  }
-}
-
-void launch_prologue(const Dev &D, int ndisks, cudaStream_t s) { k_prologue<<<1, 256, 0, s>>>(D, ndisks); }
-
-// --------------------------------------------------------------------------------------------
-// exact total barycentric momentum P_d = sum m_i v_i of every system: MOM_CTAS CTAs per system
-// accumulate their share in the lanes' integer windows, join them in shared-memory digits, add the
-// digits to the system's global accumulator, and a second pass rounds it and clears it for the next
-// use.  (Straight into the digits, 32 lanes met at the same three: the accumulation took 29, 43 and
-// 64 us for 100, 1,000 and 10,000 bodies and takes 7, 8 and 11; the rounding after it takes 5 to 6.)
+// exact total barycentric momentum P_d = sum m_i v_i of every system, in the lanes' integer windows
+// (straight into the accumulator's digits, 32 lanes met at the same three: the accumulation took 29,
+// 43 and 64 us for 100, 1,000 and 10,000 bodies and takes 7, 8 and 11).
+//   - Systems of at most MOM_ONE_MAX bodies: one CTA per system sums, rounds and, at the end of a step,
+//     drifts (k_momentum_one): 10 us for 100 bodies and 14 for 1,000, against 16 for the three kernels
+//     below; equal at 2,000.
+//   - Larger ones: MOM_CTAS CTAs per system join their sums in the system's global accumulator, a
+//     second kernel rounds it and clears it for the next use, and the drift is a third.
 // --------------------------------------------------------------------------------------------
 #define MOM_CTAS 24
+#define MOM_ONE_MAX 2048
 
-__global__ void __launch_bounds__(256) k_momentum_acc(Dev D) {
-  const int d = blockIdx.y;
-  const DiskDesc &dd = D.disks[d];
-  if (!dd.active) return;
-  __shared__ unsigned long long acc[3][SA_NDIG + 1];
-  for (int k = threadIdx.x; k < 3 * (SA_NDIG + 1); k += blockDim.x) (&acc[0][0])[k] = 0ull;
-  __syncthreads();
+// adds m v of bodies first, first + stride, ... (first: the warp's first body) to the digits in shared memory
+__device__ __forceinline__ void momentum_sum(const Dev &D, const DiskDesc &dd, int first, int stride,
+                                             unsigned long long (*acc)[SA_NDIG + 1]) {
   const int n = dd.n, off = dd.off, lane = threadIdx.x & 31;
   Window w[3];
   for (int c = 0; c < 3; ++c) win_clear(w[c]);
   int terms = 0;
-  for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
+  for (int i0 = first; i0 < n; i0 += stride) {
     const int p = off + i0 + lane;
     const double mi = i0 + lane < n && D.alive[p] ? D.m[p] : 0.0;
     const bool use = mi != 0.0;
@@ -219,6 +208,47 @@ __global__ void __launch_bounds__(256) k_momentum_acc(Dev D) {
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) win_flush(w[c], acc[c]);
+}
+
+// sun drift h = tau/2: x_i = x_i + h (P / m0), component by component (q = P_c / m0, d = h q); the shift
+// is the same for every body of a system and formed once
+__device__ __forceinline__ double sun_shift(const DiskDesc &dd, double P) {
+  return __dmul_rn(0.5 * dd.dt, __ddiv_rn(P, dd.m0));
+}
+
+__global__ void __launch_bounds__(1024) k_momentum_one(Dev D, int drift) {
+  const int d = blockIdx.x, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const DiskDesc &dd = D.disks[d];
+  if (!dd.active) return;
+  __shared__ unsigned long long acc[3][SA_NDIG + 1];
+  __shared__ double shift[3];
+  for (int k = threadIdx.x; k < 3 * (SA_NDIG + 1); k += blockDim.x) (&acc[0][0])[k] = 0ull;
+  __syncthreads();
+  momentum_sum(D, dd, threadIdx.x - lane, blockDim.x, acc);
+  __syncthreads();
+  if (wp < 3) {
+    const double r = sa_round_warp(acc[wp], lane);
+    if (lane == 0) { shift[wp] = sun_shift(dd, r); D.P[3 * d + wp] = r; }
+  }
+  if (!drift) return;
+  __syncthreads();
+  for (int i = threadIdx.x; i < dd.n; i += blockDim.x) {
+    const int p = dd.off + i;
+    if (!D.alive[p]) continue;
+    D.x[p] = __dadd_rn(D.x[p], shift[0]);
+    D.y[p] = __dadd_rn(D.y[p], shift[1]);
+    D.z[p] = __dadd_rn(D.z[p], shift[2]);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_momentum_acc(Dev D) {
+  const int d = blockIdx.y;
+  const DiskDesc &dd = D.disks[d];
+  if (!dd.active) return;
+  __shared__ unsigned long long acc[3][SA_NDIG + 1];
+  for (int k = threadIdx.x; k < 3 * (SA_NDIG + 1); k += blockDim.x) (&acc[0][0])[k] = 0ull;
+  __syncthreads();
+  momentum_sum(D, dd, blockIdx.x * blockDim.x + threadIdx.x - (threadIdx.x & 31), gridDim.x * blockDim.x, acc);
   __syncthreads();
   unsigned long long *g = D.sacc + (size_t)d * 3 * (SA_NDIG + 1);
   for (int k = threadIdx.x; k < 3 * (SA_NDIG + 1); k += blockDim.x) {
@@ -227,42 +257,46 @@ __global__ void __launch_bounds__(256) k_momentum_acc(Dev D) {
   }
 }
 
-__global__ void k_momentum_round(Dev D) {
-  const int d = blockIdx.x;
+__global__ void __launch_bounds__(96) k_momentum_round(Dev D) {
+  const int d = blockIdx.x, lane = threadIdx.x & 31, c = threadIdx.x >> 5;
   if (!D.disks[d].active) return;
   unsigned long long *g = D.sacc + (size_t)d * 3 * (SA_NDIG + 1);
-  if (threadIdx.x < 3) D.P[3 * d + threadIdx.x] = sa_round(g + threadIdx.x * (SA_NDIG + 1));
+  const double r = sa_round_warp(g + c * (SA_NDIG + 1), lane);
+  if (lane == 0) D.P[3 * d + c] = r;
   __syncthreads();
   for (int k = threadIdx.x; k < 3 * (SA_NDIG + 1); k += blockDim.x) g[k] = 0ull;
 }
 
-void launch_momentum(const Dev &D, int ndisks, cudaStream_t s) {
-  if (ndisks <= 0) return;
-  k_momentum_acc<<<dim3(MOM_CTAS, ndisks), 256, 0, s>>>(D);
-  k_momentum_round<<<ndisks, 32, 0, s>>>(D);
-}
-
 // --------------------------------------------------------------------------------------------
-// sun drift h = tau/2: x_i = x_i + h (P / m0), component by component (q = P_c / m0, d = h q).
-// The drift that opens a step also writes the FP32 copies the encounter prefilter reads.
+// sun drift.  The one that opens a step also writes the FP32 copies the encounter prefilter reads and
+// resets the per-step counters (read by later kernels only).
 // --------------------------------------------------------------------------------------------
-__global__ void k_sundrift(Dev D, long long npart, int pre) {
+template <bool OPEN>
+__global__ void k_sundrift(Dev D, long long npart, int ndisks) {
+  if (OPEN && blockIdx.x == 0) {
+    const int t = threadIdx.x;
+    if (t < 4) D.work[t] = 0;
+    if (t == 0) *D.rec_total = 0;
+    for (int d = t; d < ndisks; d += blockDim.x) {
+      D.stat[d].npairs = 0;
+      D.stat[d].ngroups = 0;
+    }
+  }
+  const int lane = threadIdx.x & 31;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npart;
-       p += (long long)gridDim.x * blockDim.x) {
+       p += (long long)gridDim.x * blockDim.x) {                 // (a warp has one 32-body block)
     const int d = D.blk_disk[p >> 5];
     if (d < 0) continue;
     const DiskDesc &dd = D.disks[d];
     if (!dd.active) continue;
+    const double q = lane < 3 ? sun_shift(dd, D.P[3 * d + lane]) : 0.0;
+    const double sx = __shfl_sync(0xffffffffu, q, 0), sy = __shfl_sync(0xffffffffu, q, 1), sz = __shfl_sync(0xffffffffu, q, 2);
     double x = D.x[p], y = D.y[p], z = D.z[p];
     if (D.alive[p]) {
-      const double h = 0.5 * dd.dt;
-      const double *P = D.P + 3 * d;
-      x = __dadd_rn(x, __dmul_rn(h, __ddiv_rn(P[0], dd.m0)));
-      y = __dadd_rn(y, __dmul_rn(h, __ddiv_rn(P[1], dd.m0)));
-      z = __dadd_rn(z, __dmul_rn(h, __ddiv_rn(P[2], dd.m0)));
+      x = __dadd_rn(x, sx); y = __dadd_rn(y, sy); z = __dadd_rn(z, sz);
       D.x[p] = x; D.y[p] = y; D.z[p] = z;
     }
-    if (pre) {
+    if (OPEN) {
       const double vx = D.vx[p], vy = D.vy[p], vz = D.vz[p];
       const float fx = __double2float_rn(x), fy = __double2float_rn(y), fz = __double2float_rn(z);
       D.xf[p] = fx; D.yf[p] = fy; D.zf[p] = fz;
@@ -279,11 +313,21 @@ __global__ void k_sundrift(Dev D, long long npart, int pre) {
   }
 }
 
-void launch_sundrift(const Dev &D, long long npart, int pre, cudaStream_t s) {
-  if (npart <= 0) return;
-  long long blocks = (npart + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  k_sundrift<<<(int)blocks, 256, 0, s>>>(D, npart, pre);
+static int sundrift_blocks(long long npart) { return (int)std::max(1LL, std::min((npart + 255) / 256, 4096LL)); }
+
+void launch_open(const Dev &D, long long npart, int ndisks, cudaStream_t s) {
+  k_sundrift<true><<<sundrift_blocks(npart), 256, 0, s>>>(D, npart, ndisks);
+}
+
+void launch_momentum(const Dev &D, int ndisks, long long npart, int n_max, bool drift, cudaStream_t s) {
+  if (ndisks <= 0) return;
+  if (n_max <= MOM_ONE_MAX) {
+    k_momentum_one<<<ndisks, std::min(1024, std::max(128, (n_max + 31) / 32 * 32)), 0, s>>>(D, drift ? 1 : 0);
+    return;
+  }
+  k_momentum_acc<<<dim3(MOM_CTAS, ndisks), 256, 0, s>>>(D);
+  k_momentum_round<<<ndisks, 96, 0, s>>>(D);
+  if (drift && npart > 0) k_sundrift<false><<<sundrift_blocks(npart), 256, 0, s>>>(D, npart, ndisks);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -298,49 +342,51 @@ __device__ __forceinline__ int macro_index(const DiskDesc &dd, int ng, int q, in
   return dd.tile_base + q * ng - (4 / SYM_MACRO_COLS) * ((q * (q - 1)) / 2) + (g - (4 / SYM_MACRO_COLS) * q);
 }
 
-__global__ void k_reduce(Dev D, long long npart) {
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npart;
-       p += (long long)gridDim.x * blockDim.x) {
-    const int d = D.blk_disk[p >> 5];
+// One CTA per 32-body block: warp w adds every RED_SLICES-th partial of the block's bodies, and the
+// sums join in warp order.  (One thread per body took 88 us for 10,000 bodies, a chain of 80 dependent
+// loads and sums on 79 CTAs; now 16 us.)
+#define RED_SLICES 8
+__global__ void __launch_bounds__(32 * RED_SLICES) k_reduce(Dev D, long long nblk) {
+  __shared__ float2 sh[RED_SLICES][3][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (long long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    const int d = D.blk_disk[blk];
     if (d < 0) continue;
     const DiskDesc &dd = D.disks[d];
     if (!dd.active) continue;
-    const int li = (int)p - dd.off;
-    if (li >= dd.n || !D.alive[p]) continue;
-    const int B = li >> 5, lane = li & 31;
+    const int B = (int)(blk - (dd.off >> 5));
     if (B >= dd.nbm) continue;                  // a block of field particles: kicked by k_field_*
     const int C = SYM_MACRO_COLS, ng = (dd.nbm + C - 1) / C, qB = B >> 2, gB = B / C;
     const int rslot = (B & 3) * 96 + lane, cslot = 384 + (B % C) * 96 + lane;
-    // the partials of p, double-float in the kick's units, in a fixed order (its rows, then its
-    // columns); two interleaved sums (even and odd terms) keep two loads in flight
+    // the partials of p, double-float in the kick's units, in a fixed order (its rows, then its columns)
     const int g0 = (4 / C) * qB, nrow = ng - g0;
     const int nterm = nrow + qB + 1;
     const float2 *part = reinterpret_cast<const float2 *>(D.part);
-    auto ptr = [&](int t) -> const float2 * {
-      if (t < nrow) return part + (size_t)macro_index(dd, ng, qB, g0 + t) * SYM_MACRO_PART + rslot;
-      const int q = t - nrow;
-      return part + (size_t)macro_index(dd, ng, q, gB) * SYM_MACRO_PART + cslot;
-    };
-    df s0[3], s1[3];
-    for (int k = 0; k < 3; ++k) s0[k] = s1[k] = mk(0.0f, 0.0f);
-    int t = 0;
-    for (; t + 1 < nterm; t += 2) {
-      const float2 *p0 = ptr(t), *p1 = ptr(t + 1);
+    df s[3];
+    for (int k = 0; k < 3; ++k) s[k] = mk(0.0f, 0.0f);
+#pragma unroll 2
+    for (int t = w; t < nterm; t += RED_SLICES) {
+      const float2 *pt = t < nrow ? part + (size_t)macro_index(dd, ng, qB, g0 + t) * SYM_MACRO_PART + rslot
+                                  : part + (size_t)macro_index(dd, ng, t - nrow, gB) * SYM_MACRO_PART + cslot;
+#pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float2 u = p0[32 * k], w = p1[32 * k];
-        s0[k] = add(s0[k], mk(u.x, u.y));
-        s1[k] = add(s1[k], mk(w.x, w.y));
+        const float2 u = pt[32 * k];
+        s[k] = add(s[k], mk(u.x, u.y));
       }
     }
-    if (t < nterm) {
-      const float2 *p0 = ptr(t);
-      for (int k = 0; k < 3; ++k) s0[k] = add(s0[k], mk(p0[32 * k].x, p0[32 * k].y));
+    for (int k = 0; k < 3; ++k) sh[w][k][lane] = make_float2(s[k].h, s[k].l);
+    __syncthreads();
+    const long long p = 32 * blk + lane;
+    if (w == 0 && (int)p - dd.off < dd.n && D.alive[p]) {
+      for (int v = 1; v < RED_SLICES; ++v)
+        for (int k = 0; k < 3; ++k) s[k] = add(s[k], mk(sh[v][k][lane].x, sh[v][k][lane].y));
+      const double h = 0.5 * dd.dt;
+      const int sc = dd.keg - 2 * dd.kex;
+      D.vx[p] = __dadd_rn(D.vx[p], __dmul_rn(h, kick_value(s[0], sc)));
+      D.vy[p] = __dadd_rn(D.vy[p], __dmul_rn(h, kick_value(s[1], sc)));
+      D.vz[p] = __dadd_rn(D.vz[p], __dmul_rn(h, kick_value(s[2], sc)));
     }
-    const double h = 0.5 * dd.dt;
-    const int sc = dd.keg - 2 * dd.kex;
-    D.vx[p] = __dadd_rn(D.vx[p], __dmul_rn(h, kick_value(add(s0[0], s1[0]), sc)));
-    D.vy[p] = __dadd_rn(D.vy[p], __dmul_rn(h, kick_value(add(s0[1], s1[1]), sc)));
-    D.vz[p] = __dadd_rn(D.vz[p], __dmul_rn(h, kick_value(add(s0[2], s1[2]), sc)));
+    __syncthreads();
   }
 }
 
@@ -388,7 +434,7 @@ void launch_reduce(const Dev &D, long long npart, int precision, cudaStream_t s)
   long long blocks = (npart + 127) / 128;
   if (blocks > 8192) blocks = 8192;
   if (precision == SYMBA_PRECISION_MIXED) k_reduce_mixed<<<(int)blocks, 128, 0, s>>>(D, npart);
-  else k_reduce<<<(int)blocks, 128, 0, s>>>(D, npart);
+  else k_reduce<<<(int)std::min(npart / 32, 65536LL), 32 * RED_SLICES, 0, s>>>(D, npart / 32);
 }
 
 // two-float split of the positions before kick 2 (mixed precision)
@@ -567,7 +613,8 @@ __global__ void __launch_bounds__(256) k_energy_pairs(Dev D, int d, unsigned lon
 }
 
 __global__ void k_energy_round(const unsigned long long *acc, double *out) {
-  if (threadIdx.x < 4) out[threadIdx.x] = sa_round(acc + threadIdx.x * (SA_NDIG + 1));
+  const double r = sa_round_warp(acc + (threadIdx.x >> 5) * (SA_NDIG + 1), threadIdx.x & 31);
+  if ((threadIdx.x & 31) == 0) out[threadIdx.x >> 5] = r;
 }
 
 void launch_energy(const Dev &D, int d, const LaunchCfg &L, unsigned long long *acc, cudaStream_t s) {
@@ -576,5 +623,5 @@ void launch_energy(const Dev &D, int d, const LaunchCfg &L, unsigned long long *
 }
 
 void launch_energy_round(unsigned long long *acc, double *out4, cudaStream_t s) {
-  k_energy_round<<<1, 32, 0, s>>>(acc, out4);
+  k_energy_round<<<1, 128, 0, s>>>(acc, out4);
 }

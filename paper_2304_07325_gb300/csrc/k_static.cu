@@ -131,19 +131,28 @@ __global__ void __launch_bounds__(256) k_static_pairs(int n, int nm, const doubl
 
 // |P|^2 / (2 m0) with P rounded from its exact sums, then E, L rounded into out[0..3]
 __global__ void k_static_finish(double m0, unsigned long long *acc, double *out) {
-  // each rounding is one thread's serial walk over the digits: side by side in the lanes
-  const int k = threadIdx.x;
-  double r = 0.0;
-  if (k >= 1 && k < STATIC_ACCS) r = sa_round(acc + k * (SA_NDIG + 1));
-  const double Px = __shfl_sync(0xffffffffu, r, 4);
-  const double Py = __shfl_sync(0xffffffffu, r, 5);
-  const double Pz = __shfl_sync(0xffffffffu, r, 6);
-  if (k == 0) {
-    const double P2 = __dadd_rn(__dadd_rn(__dmul_rn(Px, Px), __dmul_rn(Py, Py)), __dmul_rn(Pz, Pz));
-    sa_add(acc, __ddiv_rn(P2, __dmul_rn(2.0, m0)));
-    r = sa_round(acc);
+  // a warp per sum
+  __shared__ double sum[STATIC_ACCS];
+  __shared__ unsigned long long e[SA_NDIG + 1];
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (c > 0) {
+    const double r = sa_round_warp(acc + c * (SA_NDIG + 1), lane);
+    if (lane == 0) sum[c] = r;
   }
-  if (k < 4) out[k] = r;
+  __syncthreads();
+  if (c == 0) {
+    for (int k = lane; k < SA_NDIG + 1; k += 32) e[k] = acc[k];
+    __syncwarp();
+    if (lane == 0) {
+      const double P2 = __dadd_rn(__dadd_rn(__dmul_rn(sum[4], sum[4]), __dmul_rn(sum[5], sum[5])), __dmul_rn(sum[6], sum[6]));
+      sa_add(e, __ddiv_rn(P2, __dmul_rn(2.0, m0)));
+    }
+    __syncwarp();
+    const double r = sa_round_warp(e, lane);
+    if (lane == 0) out[0] = r;
+  } else if (c < 4 && lane == 0) {
+    out[c] = sum[c];
+  }
 }
 
 extern "C" int symba_energy_static(int n, int n_massive, const double *x, const double *v,
@@ -165,6 +174,6 @@ extern "C" int symba_energy_static(int n, int n_massive, const double *x, const 
   const int bb = (int)std::min<long long>((n + 255) / 256, 64);
   k_static_bodies<<<bb, 256, 0, s>>>(n, x, v, m, G, m0, acc);
   if (n_massive > 0) k_static_pairs<<<sms * 4, 256, 0, s>>>(n, n_massive, x, m, G, acc);
-  k_static_finish<<<1, 32, 0, s>>>(m0, acc, out);
+  k_static_finish<<<1, 32 * STATIC_ACCS, 0, s>>>(m0, acc, out);
   return cudaGetLastError() == cudaSuccess ? SYMBA_OK : SYMBA_E_CUDA;
 }
