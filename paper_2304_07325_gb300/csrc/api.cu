@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -105,6 +106,9 @@ struct symba_pool {
   int rec_bpsm = 1;
   int group_order = 0;
   bool any_discard = false;   // some system has a removal distance: the step runs k_discard
+  // held while work that uses the recursion's scratch is enqueued: a step, or a read that stages in it
+  std::mutex scratch;
+  std::vector<char> host;     // a small read's arrays on the host (at most READ_PACK bytes)
 };
 
 struct symba_ctx {
@@ -120,15 +124,24 @@ namespace {
     if (e_ != cudaSuccess) return SYMBA_E_CUDA;     \
   } while (0)
 
-template <class T>
-int dalloc(symba_pool *P, T **ptr, size_t count) {
-  void *p = nullptr;
-  if (count == 0) count = 1;
-  if (cudaMalloc(&p, count * sizeof(T)) != cudaSuccess) return SYMBA_E_NOMEM;
-  P->allocs.push_back(p);
-  *ptr = (T *)p;
-  return SYMBA_OK;
-}
+// A pool's device arrays are one allocation, laid out from this list: about 85 allocations and as many
+// frees, each of which waits for the device, were most of the life of a small system.
+struct Arena {
+  std::vector<std::pair<void **, size_t>> at;
+  size_t bytes = 0;
+  template <class T>
+  void add(T **ptr, size_t count) {
+    at.emplace_back((void **)ptr, bytes);
+    bytes += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
+  }
+  int allocate(symba_pool *P) {
+    void *base = nullptr;
+    if (cudaMalloc(&base, bytes) != cudaSuccess) return SYMBA_E_NOMEM;
+    P->allocs.push_back(base);
+    for (auto &r : at) *r.first = (char *)base + r.second;
+    return SYMBA_OK;
+  }
+};
 
 // a device array of the current device (or managed memory): used in place
 bool is_device_ptr(const void *p) { return pointer_class(p) == PTR_DEVICE; }
@@ -270,6 +283,7 @@ int pool_profile(symba_pool *P, int nsteps, double *phase_ms) {
   for (int k = 0; k < SYMBA_NPHASES; ++k) phase_ms[k] = 0.0;
   if (nsteps == 0 || P->ndisks == 0) return SYMBA_OK;
   CK(cudaSetDevice(P->device));
+  std::lock_guard<std::mutex> lock(P->scratch);
   cudaEvent_t ev[SYMBA_NPHASES + 1];
   for (int k = 0; k <= SYMBA_NPHASES; ++k) CK(cudaEventCreate(&ev[k]));
   k_reset_call<<<1, 256, 0, P->stream>>>(P->D.stat, P->ndisks);
@@ -319,6 +333,7 @@ int pool_step(symba_pool *P, int nsteps) {
   if (nsteps < 0) return SYMBA_E_INVAL;
   if (nsteps == 0 || P->ndisks == 0) return SYMBA_OK;
   CK(cudaSetDevice(P->device));
+  std::lock_guard<std::mutex> lock(P->scratch);
   k_reset_call<<<1, 256, 0, P->stream>>>(P->D.stat, P->ndisks);
   if (P->use_graph && !P->graph_ok) {
     cudaStreamCaptureStatus cs;
@@ -376,8 +391,8 @@ int pool_create(symba_pool **out, int max_disks, long long max_particles, long l
   }
   const long long n = P->pcap, pc = P->paircap, gs = n / 2 + 1;
   Dev &D = P->D;
-  int st = SYMBA_OK;
-  auto A = [&](auto **ptr, size_t cnt) { if (st == SYMBA_OK) st = dalloc(P, ptr, cnt); };
+  Arena arena;
+  auto A = [&](auto **ptr, size_t cnt) { arena.add(ptr, cnt); };
   A(&D.x, n); A(&D.y, n); A(&D.z, n); A(&D.vx, n); A(&D.vy, n); A(&D.vz, n);
   A(&D.m, n); A(&D.gm, n); A(&D.rad, n); A(&D.rh, n);
   A(&D.alive, n); A(&D.gid, n);
@@ -404,6 +419,7 @@ int pool_create(symba_pool **out, int max_disks, long long max_particles, long l
   A(&D.g_moff, gs); A(&D.g_mcnt, gs); A(&D.g_poff, gs); A(&D.g_pcnt, gs); A(&D.g_cur, gs);
   A(&D.gmem, n); A(&D.rec_items, gs); A(&D.rec_total, 1);
   A(&P->eacc, 4 * (SA_NDIG + 1)); A(&P->eout, 4);
+  const int st = arena.allocate(P);
   if (st != SYMBA_OK) { symba_pool_free(P); return st; }
   if (cudaMemsetAsync(D.blk_disk, 0xFF, sizeof(int) * (n / SYM_TILE + 1), P->stream) != cudaSuccess ||
       cudaMemsetAsync(D.disks, 0, sizeof(DiskDesc) * max_disks, P->stream) != cudaSuccess ||
@@ -478,10 +494,7 @@ int read_stat(symba_pool *P, int d, DiskStat *out) {
   return SYMBA_OK;
 }
 
-int slot_status(symba_pool *P, int d) {
-  DiskStat st;
-  int r = read_stat(P, d, &st);
-  if (r != SYMBA_OK) return r;
+int status_of(symba_pool *P, int d, const DiskStat &st) {
   if (st.status != 0) return st.status;
   Slot &s = P->slots[d];
   if ((long long)st.merges > s.merges_reported) {
@@ -491,40 +504,69 @@ int slot_status(symba_pool *P, int d) {
   return SYMBA_OK;
 }
 
+int slot_status(symba_pool *P, int d) {
+  DiskStat st;
+  const int r = read_stat(P, d, &st);
+  return r == SYMBA_OK ? status_of(P, d, st) : r;
+}
+
 bool valid_slot(symba_pool *P, int d) { return P && d >= 0 && d < P->max_disks && P->slots[d].active; }
 
+// Host arrays are gathered in the force slots of the recursion (D.pf), which nothing else uses and which
+// the stream has free between steps, and where those are too few in an allocation of this call.  Small
+// reads cross in one copy, large ones straight into the caller's arrays; the status comes with them,
+// so a read waits for the device once.
+#define READ_PACK (256 << 10)
 int get_state(symba_pool *P, int d, double *x, double *v, double *m, double *rad, int *alive) {
   if (!valid_slot(P, d)) return SYMBA_E_INVAL;
   CK(cudaSetDevice(P->device));
   const int n = P->slots[d].n;
   if (is_foreign_ptr(x) || is_foreign_ptr(v) || is_foreign_ptr(m) || is_foreign_ptr(rad) || is_foreign_ptr(alive))
     return SYMBA_E_INVAL;
-  double *dx = nullptr, *dv = nullptr, *dm = nullptr, *dr = nullptr;
-  int *da = nullptr;
-  const bool hx = x && !is_device_ptr(x), hv = v && !is_device_ptr(v), hm = m && !is_device_ptr(m),
-             hr = rad && !is_device_ptr(rad), ha = alive && !is_device_ptr(alive);
-  int st = SYMBA_OK;
-  auto tmp = [&](bool need, void **pp, size_t bytes) {
-    if (need && st == SYMBA_OK && cudaMalloc(pp, bytes) != cudaSuccess) st = SYMBA_E_NOMEM;
-  };
-  tmp(hx, (void **)&dx, sizeof(double) * 3 * n);
-  tmp(hv, (void **)&dv, sizeof(double) * 3 * n);
-  tmp(hm, (void **)&dm, sizeof(double) * n);
-  tmp(hr, (void **)&dr, sizeof(double) * n);
-  tmp(ha, (void **)&da, sizeof(int) * n);
-  if (st == SYMBA_OK) {
-    launch_gather_state(P->D, d, n, hx ? dx : x, hv ? dv : v, hm ? dm : m, hr ? dr : rad, ha ? da : alive,
-                        nullptr, P->stream);
-    if (hx) cudaMemcpyAsync(x, dx, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, P->stream);
-    if (hv) cudaMemcpyAsync(v, dv, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, P->stream);
-    if (hm) cudaMemcpyAsync(m, dm, sizeof(double) * n, cudaMemcpyDeviceToHost, P->stream);
-    if (hr) cudaMemcpyAsync(rad, dr, sizeof(double) * n, cudaMemcpyDeviceToHost, P->stream);
-    if (ha) cudaMemcpyAsync(alive, da, sizeof(int) * n, cudaMemcpyDeviceToHost, P->stream);
-    if (cudaStreamSynchronize(P->stream) != cudaSuccess) st = SYMBA_E_CUDA;
+  struct Part {
+    void *user, *dev;
+    size_t bytes, at;
+    bool host;
+  } part[5] = {{x, x, sizeof(double) * 3 * n, 0, false}, {v, v, sizeof(double) * 3 * n, 0, false},
+               {m, m, sizeof(double) * n, 0, false}, {rad, rad, sizeof(double) * n, 0, false},
+               {alive, alive, sizeof(int) * n, 0, false}};
+  size_t total = 0;
+  for (Part &q : part) {
+    q.host = q.user && !is_device_ptr(q.user);
+    if (!q.host) continue;
+    q.at = total;
+    total += (q.bytes + 15) / 16 * 16;
   }
-  cudaFree(dx); cudaFree(dv); cudaFree(dm); cudaFree(dr); cudaFree(da);
-  if (st != SYMBA_OK) return st;
-  return slot_status(P, d);
+  DiskStat stat;
+  void *own = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(P->scratch);
+    char *stage = (char *)P->D.pf;
+    if (total > sizeof(double) * 5 * (size_t)P->paircap) {
+      if (cudaMalloc(&own, total) != cudaSuccess) return SYMBA_E_NOMEM;
+      stage = (char *)own;
+    }
+    for (Part &q : part)
+      if (q.host) q.dev = stage + q.at;
+    launch_gather_state(P->D, d, n, (double *)part[0].dev, (double *)part[1].dev, (double *)part[2].dev,
+                        (double *)part[3].dev, (int *)part[4].dev, nullptr, P->stream);
+    const bool pack = total <= READ_PACK;
+    bool ok = true;
+    if (pack && total) {
+      if (P->host.size() < total) P->host.resize(total);
+      ok = cudaMemcpyAsync(P->host.data(), stage, total, cudaMemcpyDeviceToHost, P->stream) == cudaSuccess;
+    }
+    for (const Part &q : part)
+      if (!pack && q.host && cudaMemcpyAsync(q.user, q.dev, q.bytes, cudaMemcpyDeviceToHost, P->stream) != cudaSuccess) ok = false;
+    if (cudaMemcpyAsync(&stat, P->D.stat + d, sizeof(stat), cudaMemcpyDeviceToHost, P->stream) != cudaSuccess) ok = false;
+    if (cudaStreamSynchronize(P->stream) != cudaSuccess) ok = false;
+    if (own) cudaFree(own);
+    if (!ok) return SYMBA_E_CUDA;
+    if (pack)
+      for (const Part &q : part)
+        if (q.host) memcpy(q.user, P->host.data() + q.at, q.bytes);
+  }
+  return status_of(P, d, stat);
 }
 
 int get_rhill(symba_pool *P, int d, double *rh) {
