@@ -8,7 +8,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -108,7 +110,7 @@ struct symba_pool {
   bool any_discard = false;   // some system has a removal distance: the step runs k_discard
   // held while work that uses the recursion's scratch is enqueued: a step, or a read that stages in it
   std::mutex scratch;
-  std::vector<char> host;     // a small read's arrays on the host (at most READ_PACK bytes)
+  std::unique_ptr<char[]> host;   // a small read's arrays on the host (READ_PACK bytes)
 };
 
 struct symba_ctx {
@@ -550,12 +552,10 @@ int get_state(symba_pool *P, int d, double *x, double *v, double *m, double *rad
       if (q.host) q.dev = stage + q.at;
     launch_gather_state(P->D, d, n, (double *)part[0].dev, (double *)part[1].dev, (double *)part[2].dev,
                         (double *)part[3].dev, (int *)part[4].dev, nullptr, P->stream);
-    const bool pack = total <= READ_PACK;
+    if (total && total <= READ_PACK && !P->host) P->host.reset(new (std::nothrow) char[READ_PACK]);
+    const bool pack = total <= READ_PACK && P->host;
     bool ok = true;
-    if (pack && total) {
-      if (P->host.size() < total) P->host.resize(total);
-      ok = cudaMemcpyAsync(P->host.data(), stage, total, cudaMemcpyDeviceToHost, P->stream) == cudaSuccess;
-    }
+    if (pack && total) ok = cudaMemcpyAsync(P->host.get(), stage, total, cudaMemcpyDeviceToHost, P->stream) == cudaSuccess;
     for (const Part &q : part)
       if (!pack && q.host && cudaMemcpyAsync(q.user, q.dev, q.bytes, cudaMemcpyDeviceToHost, P->stream) != cudaSuccess) ok = false;
     if (cudaMemcpyAsync(&stat, P->D.stat + d, sizeof(stat), cudaMemcpyDeviceToHost, P->stream) != cudaSuccess) ok = false;
@@ -564,7 +564,7 @@ int get_state(symba_pool *P, int d, double *x, double *v, double *m, double *rad
     if (!ok) return SYMBA_E_CUDA;
     if (pack)
       for (const Part &q : part)
-        if (q.host) memcpy(q.user, P->host.data() + q.at, q.bytes);
+        if (q.host) memcpy(q.user, P->host.get() + q.at, q.bytes);
   }
   return status_of(P, d, stat);
 }

@@ -42,7 +42,8 @@ def test_reads_beside_steps_of_another_thread():
     ds = [disk.planetesimal_disk(400, 80 + k) for k in range(2)]
     tiles = sum(((d.n + 31) // 32) ** 2 for d in ds)
     pool = sy.Pool(2, sum(d.n for d in ds), tiles)
-    slots = [pool.admit(d.x, d.v, d.m, d.radius) for d in ds]
+    params = sy.default_params(dt=0.01, hill_scale=0.0)          # no encounters, so no mergers
+    slots = [pool.admit(d.x, d.v, d.m, d.radius, params=params) for d in ds]
     bad = []
 
     def read():
