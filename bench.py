@@ -29,18 +29,20 @@ import numpy as np  # noqa: E402
 
 FLOPS_PER_PAIR_KICK = 26          # 3 sub, 5 r^2, 2 for 1/sqrt, 2 for r^-3, 2 mass scalings, 12 FMA flops
 FLOPS_PER_PAIR_CHECK = 18
-# FP64 warp instructions of the group recursion per sub-step, by path: least-squares fit of ncu's
-# smsp__inst_executed_pipe_fp64.sum per k_recursion launch against the launches' per-path sub-step
-# counts over four steps of the N = 10,000 disk (residuals <= 1.1 %; profiles/k_recursion_fp64_fit.md).
-# A general sub-step of a large group covers every body and pair of the group.
-FP64_PER_PAIR_SUBSTEP = 21.70
-FP64_PER_GENERAL_SUBSTEP = 936.0
+# Warp instructions of the group recursion per sub-step, by path: least-squares fit of ncu's
+# smsp__inst_executed.sum per k_recursion launch against the launches' per-path sub-step counts over
+# four steps of the N = 10,000 disk (residuals <= 1.0 %; profiles/k_recursion_disk_N10000.md).  A general
+# sub-step covers every body and pair of the group at its level.
+INSTR_PER_PAIR_SUBSTEP = 335.9
+INSTR_PER_GENERAL_SUBSTEP = 4942.7
+# and of the FP64 pair kick per pair: mean of kick 1 and kick 2 (profiles/k_trap_df_disk_N10000.md)
+INSTR_PER_PAIR_KICK = (428516403 + 388191833) / 2 / 49995000
 # The recursion of the bound-pair group the profiles use (bodies of the N = 10,000 disk, seed 1002)
 BOUND_PAIR_GROUP = [1244, 3406, 4643, 5122, 9870]
 # DRAM read + write per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum, N = 10,000, FP64)
 # of the current kernels; None until a capture of the current kernel is on record
-RECURSION_TRAFFIC_BYTES = 1987840 + 19968      # first step of the disk (profiles/k_recursion_fp64_fit.md)
-KICK_TRAFFIC_BYTES = ((1148928 + 0) + (725248 + 256)) / 2        # kick 1, kick 2 (profiles/k_trap_fp64_disk_N10000.md)
+RECURSION_TRAFFIC_BYTES = 1388288 + 6144       # first step of the disk (profiles/k_recursion_disk_N10000.md)
+KICK_TRAFFIC_BYTES = ((1154560 + 0) + (730112 + 0)) / 2          # kick 1, kick 2 (profiles/k_trap_df_disk_N10000.md)
 # Step size at which the batched and served forms and the one-at-a-time form all keep the energy
 # error of every merger-free disk below 1e-10 (measured on the 64 batched disks: 5.7e-11 after 20
 # steps at 0.125 yr, 1.1e-10 at 0.2, 5.2e-10 at 0.5)
@@ -626,40 +628,42 @@ def run_ours(args):
         fp64_tflops = rates["fp64_flops"] / 1e12
         rec_s = phase_tot[5] * 1e-3
         sm_hz = 1e6 * (clk.get("sm_mhz") or 2070.0)
-        # the dominant kernel: the group recursion.  Its FP64 warp instructions per step are the
-        # run's own per-path sub-step counts times the per-path counts ncu measured
+        # the dominant kernel: the group recursion.  Its warp instructions per step are the run's own
+        # per-path sub-step counts times the per-path counts ncu measured; the peak is one instruction
+        # per scheduler and cycle
         gen_substeps = substeps - pair_substeps
-        fp64_instr = FP64_PER_PAIR_SUBSTEP * pair_substeps + FP64_PER_GENERAL_SUBSTEP * gen_substeps
-        chip_peak = rates["fp64_flops"] / 64.0          # FP64 warp instructions/s (32 lanes x 2 flops)
-        rec_achieved = fp64_instr / rec_s if rec_s > 0 else 0.0
+        rec_instr = INSTR_PER_PAIR_SUBSTEP * pair_substeps + INSTR_PER_GENERAL_SUBSTEP * gen_substeps
+        chip_peak = 4.0 * rates["sms"] * sm_hz
+        rec_achieved = rec_instr / rec_s if rec_s > 0 else 0.0
         chain_us = statistics.median(chain_us_list) if chain_us_list else float("nan")
-        chain_peak = sm_hz / rates["warp_dfma_dep_cycles"]                # one warp, FP64 instr/s
-        chain_achieved = FP64_PER_PAIR_SUBSTEP / (chain_us * 1e-6)
+        chain_achieved = INSTR_PER_PAIR_SUBSTEP / (chain_us * 1e-6)
         traffic_ok = args.n == 10000 and args.n_field == 0 and prec == 0
-        roofline = {"kernel": "k_recursion (per-group recursive sub-stepping)", "bound": "alu",
-                    "achieved": rec_achieved, "peak": chip_peak, "unit": "FP64 warp-instructions/s",
+        peak_source = "4 schedulers x SMs x the SM clock sampled in this run, one warp instruction per cycle"
+        roofline = {"kernel": "k_recursion (per-group recursive sub-stepping)", "bound": "latency",
+                    "achieved": rec_achieved, "peak": chip_peak, "unit": "warp-instructions/s",
                     "frac": rec_achieved / chip_peak, "traffic": RECURSION_TRAFFIC_BYTES if traffic_ok else None,
                     "share_of_step": phase_tot[5] / phase_tot.sum(),
-                    "peak_source": f"measured by symba_measure_rates in this run: {fp64_tflops:.4f} TFLOP/s FP64 "
-                                   "(independent FMAs on every SM) / 64 flops per warp instruction",
-                    "fp64_instr_per_step": fp64_instr / args.steps,
-                    "fp64_instr_model": f"{FP64_PER_PAIR_SUBSTEP} per single-pair sub-step x {pair_substeps} + "
-                                        f"{FP64_PER_GENERAL_SUBSTEP} per general sub-step x {gen_substeps} "
-                                        "(this run's counts; per-path figures from ncu, "
-                                        "profiles/k_recursion_fp64_fit.md)",
-                    "chain": {"what": "the longest group's dependent chain on one warp against one warp's FP64 "
-                                      "issue (one instruction per warp_dfma_dep_cycles, measured)",
-                              "achieved": chain_achieved, "peak": chain_peak, "unit": "FP64 instr/s, one warp",
-                              "frac": chain_achieved / chain_peak, "us_per_chain_substep": chain_us,
+                    "peak_source": peak_source,
+                    "instr_per_step": rec_instr / args.steps,
+                    "instr_model": f"{INSTR_PER_PAIR_SUBSTEP} per single-pair sub-step x {pair_substeps} + "
+                                   f"{INSTR_PER_GENERAL_SUBSTEP} per general sub-step x {gen_substeps} "
+                                   "(this run's counts; per-path figures from ncu, "
+                                   "profiles/k_recursion_disk_N10000.md)",
+                    "chain": {"what": "the longest group's dependent chain on one warp against one warp's issue "
+                                      "(one instruction per cycle)",
+                              "achieved": chain_achieved, "peak": sm_hz, "unit": "warp-instructions/s, one warp",
+                              "frac": chain_achieved / sm_hz, "us_per_chain_substep": chain_us,
                               "warp_dfma_dep_cycles": rates["warp_dfma_dep_cycles"]},
                     "note": "latency-bound: each group's sub-steps are one dependent chain on one warp, and the "
-                            "longest chain sets the step time, so most of the chip's FP64 lanes idle"}
-        roofline_kick = {"kernel": "k_trap_fp64 (trapezoid pair kick)", "bound": "alu", "achieved": kick_tflops,
-                         "peak": fp64_tflops, "unit": "TFLOP/s", "frac": kick_tflops / fp64_tflops,
+                            "longest chain sets the step time, so most of the chip's schedulers idle"}
+        kick_instr = INSTR_PER_PAIR_KICK * P / (kick_ms * 1e-3) if prec == 0 else None
+        roofline_kick = {"kernel": "k_trap_df (trapezoid pair kick, double-float)" if prec == 0 else "k_trap_mixed",
+                         "bound": "alu", "achieved": kick_instr, "peak": chip_peak, "unit": "warp-instructions/s",
+                         "frac": kick_instr / chip_peak if kick_instr else None,
                          "traffic": KICK_TRAFFIC_BYTES if traffic_ok else None,
                          "algorithmic_bytes": 32 * args.n + 48 * args.n,
                          "ms_per_launch": kick_ms, "flops_per_pair": FLOPS_PER_PAIR_KICK,
-                         "peak_source": "measured by symba_measure_rates in this run (FP64 FMAs on every SM)"}
+                         "tflops": kick_tflops, "fp64_tflops": fp64_tflops, "peak_source": peak_source}
         phases = {name: phase_tot[i] / args.steps for i, name in enumerate(sy.PHASES)}
         second = None
         if args.second_n > 0 and world == 1 and args.n_field == 0 and prec == 0:
@@ -701,8 +705,8 @@ def run_ours(args):
                         "h2d_bytes_per_step": 2 * 8 * 3 * ntot, "d2h_bytes_per_step": 2 * 8 * 3 * ntot,
                         "steps": ne, "trajectory": "the timed steps' (second context, same warm-up)"
                         if ne == args.steps else f"the first {ne} of the timed steps'"},
-                # per timed step: the step's 12 kernels plus the per-call statistics reset (the
-                # loop times each step as its own call; the launch list shows the same 13)
+                # per timed step: the step's 11 kernels plus the per-call statistics reset (the
+                # loop times each step as its own call)
                 "gpu_launches": args.steps * 12,
                 "clocks": clk, "wall_s": wall, "second": second, "rates": rates,
                 "chain_vs_cpu": chain, "batched": batched, "served": served, "field": field}

@@ -8,8 +8,8 @@
         bound pair: the group recursion (k_recursion) dominates, ~34,000 sub-steps per step
     python -m paper_2304_07325_gb300.profile_cases steps --n 10000 --steps 4
         the disk stepped one call per step, with each step's recursion sub-steps split by path
-        (single-pair / general) -- beside an ncu count of FP64 instructions per k_recursion
-        launch, the FP64 instructions per sub-step of each path follow by least squares
+        (single-pair / general) -- beside an ncu count of instructions per k_recursion launch,
+        the instructions per sub-step of each path follow by least squares
 
 Each case prints the per-phase device times measured with CUDA events (symba_profile_step).
 """
