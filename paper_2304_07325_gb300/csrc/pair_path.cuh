@@ -43,12 +43,12 @@
 // Cost and bound (one GB300 at 2.07 GHz).  A cleared order-2 sub-step is ~410 warp instructions, 95 %
 // of them FP32, on a dependent path of ~500 cycles, and takes ~720; the component-packed FP64 form it
 // replaces issued 22 FP64 and ~480 other instructions in 2,360.  Recursion time over the sub-steps of
-// the longest chain, before and after: 10,000-body disk 1.12 -> 0.31 us (first step 113 -> 30 ms),
-// 5,000 1.16 -> 0.30, 1,000 + 100,000 field 1.15 -> 0.33; chains of shallow levels, where the FP64
-// Kepler solver and order-6 series cost 6 to 15 us, 4.4 -> 0.7 (1,000-body disk).
-// Error against an 80-bit integration of 380 two- and many-body systems, one step: 0.05 of the FP64
+// the longest chain, before and now: 10,000-body disk 1.12 -> 0.28 us (first step 113 -> 28 ms),
+// 5,000 1.16 -> 0.30, 1,000 + 100,000 field 1.15 -> 0.30; chains of shallow levels, where a sub-step
+// takes 0.6 us (order 6), 1.3 (order 10) or 6 to 12 (the Kepler solver), 4.4 -> 0.7 (1,000-body disk).
+// Error against an 80-bit integration of 430 two- and many-body systems, one step: 0.054 of the FP64
 // form's on the geometric mean (the separation is exact here, see above).
-// The routine is inlined into its two callers: as a function of its own the calling convention left
+// The routine is inlined into its caller: as a function of its own the calling convention left
 // the compiler too few registers to interleave the chains (0.40 against 0.26 us per sub-step).
 #include "df32.cuh"
 
