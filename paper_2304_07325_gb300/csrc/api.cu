@@ -241,8 +241,6 @@ int rebuild(symba_pool *P) {
     memcpy(descs[d].ck2, cur[d].ck2, sizeof(descs[d].ck2));
     memcpy(descs[d].invdc, cur[d].invdc, sizeof(descs[d].invdc));
     memcpy(descs[d].hk, cur[d].hk, sizeof(descs[d].hk));
-    descs[d].kex = cur[d].kex;
-    descs[d].keg = cur[d].keg;
   }
   CK(cudaMemcpyAsync(P->D.disks, descs.data(), sizeof(DiskDesc) * P->max_disks, cudaMemcpyHostToDevice, P->stream));
   invalidate_graph(P);

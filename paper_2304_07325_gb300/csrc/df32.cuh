@@ -152,5 +152,5 @@ __device__ __forceinline__ double scale2(double a, int k) {
 }
 // A sum of scaled accelerations as a double, scaled back by 2^k.
 __device__ __forceinline__ double kick_value(df a, int k) {
-  return scale2(__dadd_rn((double)a.h, (double)a.l), k);
+  return scale2(__dadd_rn(f32_to_f64(a.h), f32_to_f64(a.l)), k);
 }

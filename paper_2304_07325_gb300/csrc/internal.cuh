@@ -10,8 +10,8 @@
 //                                                    of 32 x 32 tiles (128-body quads q <= c)
 //   fblk                                           : int2 {system, block} per block of field particles
 //   part                                           : [macro-tile][rows, columns][4][3][32] pair-kick
-//                                                    partials, 8 bytes each (double-float; mixed: FP32
-//                                                    sum and compensation)
+//                                                    partials, 8 bytes each (FP64; mixed: FP32 sum and
+//                                                    compensation)
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -34,7 +34,6 @@ struct DiskDesc {
   int pair_base, pair_cap;      // this system's slice of the pair buffers
   int group_base;               // this system's slice of the group slots (= off / 2)
   int active, M, l, max_depth, max_substeps, pad0;
-  int kex, keg;                 // exponents of the kick's units: positions 2^kex, G m 2^keg (set-up)
   double dt, shell_ratio, hill_scale, G, m0;
   double rmin2, rmax2;          // squared removal distances (0 = no limit)
   double ck[SYM_MAX_LEVELS + 2];    // c_k = c_{k-1} / shell_ratio, c_0 = 1 (R_k = R_0 c_k)
@@ -66,7 +65,7 @@ struct Dev {
   unsigned long long *sacc;     // [max_disks][3][SA_NDIG + 1] exact accumulators
   // trapezoid
   int4 *tiles;                  // macro-tiles (quads q <= c) over the blocks holding massive bodies
-  double *part;                 // [macro-tile][SYM_MACRO_PART] FP32 pairs
+  double *part;                 // [macro-tile][SYM_MACRO_PART] (mixed: pairs of FP32)
   int2 *fblk;                   // field rectangle: {system, block} of every block of field particles only
   int nfblk;
   int *work;                    // [4] dynamic work counters (kick 1, kick 2, recursion, spare)

@@ -76,28 +76,21 @@ void launch_discard(const Dev &D, long long npart, cudaStream_t s) {
 // and Hill radii rH_i = a_i (m_i / 3 m0)^{1/3} from the osculating heliocentric orbit
 // (vis-viva 1/a = 2/r - v^2/mu, mu = G (m0 + m_i); r if unbound; correctly rounded cube root).
 // --------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const double *xh, const double *vh,
-                                                   const double *m, double *q_out) {
+__global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const double *vh, const double *m,
+                                                   double *q_out) {
   __shared__ unsigned long long acc[4][SA_NDIG + 1];
-  __shared__ int top[2];                  // high words of the largest |x| component and |G m|
-  if (threadIdx.x < 2) top[threadIdx.x] = 0;
   for (int k = threadIdx.x; k < 4 * (SA_NDIG + 1); k += blockDim.x) (&acc[0][0])[k] = 0ull;
   __syncthreads();
-  const double G = D.disks[d].G;
   Window w[4];
   for (int c = 0; c < 4; ++c) win_clear(w[c]);
-  int xtop = 0, gtop = 0, terms = 0;
+  int terms = 0;
   const int lane = threadIdx.x & 31;
   for (int i0 = threadIdx.x - lane; i0 < n; i0 += blockDim.x) {      // whole warps
     const int i = i0 + lane;
     const double mi = i < n ? m[i] : 0.0;
     win_add(w[3], acc[3], mi);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      win_add(w[c], acc[c], i < n ? __dmul_rn(mi, vh[3 * i + c]) : 0.0);
-      if (i < n) xtop = max(xtop, __double2hiint(xh[3 * i + c]) & 0x7FFFFFFF);
-    }
-    gtop = max(gtop, __double2hiint(__dmul_rn(G, mi)) & 0x7FFFFFFF);
+    for (int c = 0; c < 3; ++c) win_add(w[c], acc[c], i < n ? __dmul_rn(mi, vh[3 * i + c]) : 0.0);
     if (++terms == WIN_TERMS) {
       for (int c = 0; c < 4; ++c) win_flush(w[c], acc[c]);
       terms = 0;
@@ -105,9 +98,6 @@ __global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const do
   }
 #pragma unroll
   for (int c = 0; c < 4; ++c) win_flush(w[c], acc[c]);
-  xtop = __reduce_max_sync(0xffffffffu, xtop);
-  gtop = __reduce_max_sync(0xffffffffu, gtop);
-  if (lane == 0) { atomicMax(&top[0], xtop); atomicMax(&top[1], gtop); }
   __syncthreads();
   __shared__ double sum[4];
   if (threadIdx.x < 128) {
@@ -116,8 +106,6 @@ __global__ void __launch_bounds__(256) k_init_sums(Dev D, int d, int n, const do
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    D.disks[d].kex = (top[0] >> 20) - 1023;
-    D.disks[d].keg = top[1] ? (top[1] >> 20) - 1023 : 0;
     const double denom = __dadd_rn(D.disks[d].m0, sum[3]);
     for (int c = 0; c < 3; ++c) q_out[c] = __ddiv_rn(sum[c], denom);
   }
@@ -170,7 +158,7 @@ void launch_init_state(const Dev &D, int d, int n, const double *xh, const doubl
                        cudaStream_t s) {
   // q (3 doubles) lives in the momentum slot of the system until the first momentum pass
   double *q = D.P + 3 * d;
-  k_init_sums<<<1, 256, 0, s>>>(D, d, n, xh, vh, m, q);
+  k_init_sums<<<1, 256, 0, s>>>(D, d, n, vh, m, q);
   k_init_state<<<64, 256, 0, s>>>(D, d, n, xh, vh, m, rad, rh, compute_rh, q);
 }
 
@@ -347,7 +335,7 @@ __device__ __forceinline__ int macro_index(const DiskDesc &dd, int ng, int q, in
 // loads and sums on 79 CTAs; now 16 us.)
 #define RED_SLICES 8
 __global__ void __launch_bounds__(32 * RED_SLICES) k_reduce(Dev D, long long nblk) {
-  __shared__ float2 sh[RED_SLICES][3][32];
+  __shared__ double sh[RED_SLICES][3][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (long long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
     const int d = D.blk_disk[blk];
@@ -358,33 +346,25 @@ __global__ void __launch_bounds__(32 * RED_SLICES) k_reduce(Dev D, long long nbl
     if (B >= dd.nbm) continue;                  // a block of field particles: kicked by k_field_*
     const int C = SYM_MACRO_COLS, ng = (dd.nbm + C - 1) / C, qB = B >> 2, gB = B / C;
     const int rslot = (B & 3) * 96 + lane, cslot = 384 + (B % C) * 96 + lane;
-    // the partials of p, double-float in the kick's units, in a fixed order (its rows, then its columns)
+    // the partials of p in a fixed order (its rows, then its columns)
     const int g0 = (4 / C) * qB, nrow = ng - g0;
     const int nterm = nrow + qB + 1;
-    const float2 *part = reinterpret_cast<const float2 *>(D.part);
-    df s[3];
-    for (int k = 0; k < 3; ++k) s[k] = mk(0.0f, 0.0f);
+    double s[3] = {0.0, 0.0, 0.0};
 #pragma unroll 2
     for (int t = w; t < nterm; t += RED_SLICES) {
-      const float2 *pt = t < nrow ? part + (size_t)macro_index(dd, ng, qB, g0 + t) * SYM_MACRO_PART + rslot
-                                  : part + (size_t)macro_index(dd, ng, t - nrow, gB) * SYM_MACRO_PART + cslot;
+      const double *pt = t < nrow ? D.part + (size_t)macro_index(dd, ng, qB, g0 + t) * SYM_MACRO_PART + rslot
+                                  : D.part + (size_t)macro_index(dd, ng, t - nrow, gB) * SYM_MACRO_PART + cslot;
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float2 u = pt[32 * k];
-        s[k] = add(s[k], mk(u.x, u.y));
-      }
+      for (int k = 0; k < 3; ++k) s[k] += pt[32 * k];
     }
-    for (int k = 0; k < 3; ++k) sh[w][k][lane] = make_float2(s[k].h, s[k].l);
+    for (int k = 0; k < 3; ++k) sh[w][k][lane] = s[k];
     __syncthreads();
     const long long p = 32 * blk + lane;
-    if (w == 0 && (int)p - dd.off < dd.n && D.alive[p]) {
-      for (int v = 1; v < RED_SLICES; ++v)
-        for (int k = 0; k < 3; ++k) s[k] = add(s[k], mk(sh[v][k][lane].x, sh[v][k][lane].y));
-      const double h = 0.5 * dd.dt;
-      const int sc = dd.keg - 2 * dd.kex;
-      D.vx[p] = __dadd_rn(D.vx[p], __dmul_rn(h, kick_value(s[0], sc)));
-      D.vy[p] = __dadd_rn(D.vy[p], __dmul_rn(h, kick_value(s[1], sc)));
-      D.vz[p] = __dadd_rn(D.vz[p], __dmul_rn(h, kick_value(s[2], sc)));
+    if (w < 3 && (int)p - dd.off < dd.n && D.alive[p]) {      // warp w joins component w (an FP64 sum takes a warp 64 cycles)
+      double a = sh[0][w][lane];
+      for (int v = 1; v < min(RED_SLICES, nterm); ++v) a += sh[v][w][lane];
+      double *vel = w == 0 ? D.vx : (w == 1 ? D.vy : D.vz);
+      vel[p] = __dadd_rn(vel[p], __dmul_rn(0.5 * dd.dt, a));
     }
     __syncthreads();
   }

@@ -39,7 +39,7 @@
 #define FULL 0xffffffffu
 
 struct TileCtx {
-  int off, n, nm, pair_base, pair_cap, l, kex, keg;
+  int off, n, nm, pair_base, pair_cap, l;
   double dt, lam, c0, c1;
 };
 
@@ -47,7 +47,6 @@ __device__ __forceinline__ TileCtx load_ctx(const DiskDesc *dp) {
   TileCtx c;
   c.off = dp->off; c.n = dp->n; c.nm = dp->nm;
   c.pair_base = dp->pair_base; c.pair_cap = dp->pair_cap; c.l = dp->l;
-  c.kex = dp->kex; c.keg = dp->keg;
   c.dt = dp->dt; c.lam = dp->hill_scale; c.c0 = dp->ck[0]; c.c1 = dp->ck[1];
   return c;
 }
@@ -55,6 +54,16 @@ __device__ __forceinline__ TileCtx load_ctx(const DiskDesc *dp) {
 __device__ __forceinline__ double g0_weight(const TileCtx &c, double R0, double r) {
   const double Rk = R0 * c.c0, Rk1 = R0 * c.c1;
   return partition_fn((r - Rk1) / (Rk - Rk1), c.l);
+}
+
+// level-0 weight of a pair by the encounter predicate: g_0(r) when it is flagged, else 1
+__device__ __forceinline__ double flagged_weight(const Dev &D, const TileCtx &c, int lo, int hi) {
+  const double ex = __dsub_rn(D.x[hi], D.x[lo]), ey = __dsub_rn(D.y[hi], D.y[lo]), ez = __dsub_rn(D.z[hi], D.z[lo]);
+  const double evx = __dsub_rn(D.vx[hi], D.vx[lo]), evy = __dsub_rn(D.vy[hi], D.vy[lo]),
+               evz = __dsub_rn(D.vz[hi], D.vz[lo]);
+  const double R0 = __dmul_rn(c.lam, __dadd_rn(D.rh[lo], D.rh[hi]));
+  if (!encounter_exact(ex, ey, ez, evx, evy, evz, R0, c.dt)) return 1.0;
+  return g0_weight(c, R0, __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez))));
 }
 
 // Binary search of (lo, hi) in the sorted pair list of a group.
@@ -94,8 +103,8 @@ __device__ __forceinline__ void on_grid(double x, int E, int kex, float &a, floa
   b = __int2float_rn((int)((X >> 20) & 0xFFFFF)) * (sa * 9.5367432e-7f);                   // 2^-20
   c = __int2float_rn((int)(X & 0xFFFFF)) * (sa * 9.0949470e-13f);                          // 2^-40
 }
-// exponent of the grid of a component: that of its largest |x| (biased as in hi, the largest high
-// word), not below 2^-60 of the system's scale
+// exponent of the grid of a component: that of its largest |x| (hi: the largest high word), not below
+// 2^-60 of the largest of the three
 __device__ __forceinline__ int grid_exp(int hi, int kex) { return max((hi >> 20) - 1023, kex - 60); }
 __device__ __forceinline__ df separation(float aj, float bj, float cj, float ai, float bi, float ci) {
   const df t = fast_two_sum(__fsub_rn(aj, ai), __fsub_rn(bj, bi));   // |da| >= |db| or da = 0
@@ -108,6 +117,40 @@ __device__ __forceinline__ void accumulate(df &sum, df t) {
   sum.l = __fadd_rn(sum.l, __fadd_rn(s.l, t.l));
 }
 
+// ---- how far the double-float form may go
+// Positions are scaled by 2^-kex and G m by 2^-keg, the largest of the macro-tile (of the field chunk), so
+// neither what lies elsewhere in the system nor how far it has spread since set-up matters.  What is lost:
+// the grid moves a separation by up to sqrt(3) 2^-61, which changes a pair's force s d (s = G m / r^3) by
+// up to 4 sqrt(3) 2^-61 s < 2^-58 s.  Every body's sum of s GRID_TERM 2^-46 is kept beside its force and
+// the macro-tile is taken again in FP64 (macro_general) when, times tau/2, it may exceed 2^-54 |v| of a
+// body -- half of what the rounding of v loses anyway -- or when a force left the FP32 range.  So a body far
+// from the rest (ejected, or parked) costs the macro-tiles it is in time and not accuracy: for pairs 0.05 AU
+// apart in a disk of 10 AU the double-float force is off by 2e-16 of itself, and with a body of the
+// macro-tile at 1e8 AU by 1.5e-9.
+#define GRID_TERM 2.4414062e-4f          // 2^-12
+struct Units {
+  int kex, keg;
+  bool fits;             // the exponents leave room for the scaled arithmetic
+};
+__device__ __forceinline__ int top_exp(int hi) { return (hi >> 20) - 1023; }
+// from the high words of the largest |x|, |y|, |z|, G m and the smallest G m > 0
+__device__ __forceinline__ Units units_of(int hx, int hy, int hz, int gmax, int gmin) {
+  Units u;
+  u.kex = top_exp(max(hx, max(hy, hz)));
+  u.keg = gmax ? top_exp(gmax) : 0;
+  // (a G m below 2^-80 of the largest would lose its low part)
+  u.fits = abs(u.kex) <= 250 && abs(u.keg) <= 250 && (gmax == 0 || top_exp(gmin) >= u.keg - 80);
+  return u;
+}
+// Largest sum of s GRID_TERM (scaled) allowed for a body: 2^-8 |v| / (tau/2) over the square root of the
+// number of such sums (their errors are independent), rounded down to a power of two.  hv: high word of
+// the body's largest |v| component.
+__device__ __forceinline__ float error_room(int hv, double dt, const Units &u, int nsum) {
+  const int eh = top_exp(__double2hiint(dt) & 0x7FFFFFFF);          // tau/2 < 2^eh
+  const int n = top_exp(hv) - 8 - eh + 2 * u.kex - u.keg - (33 - __clz(nsum)) / 2;
+  return n < -126 ? 0.0f : __int_as_float(min(n + 127, 254) << 23);
+}
+
 // the row side of one warp: row particle I*32 + lane, its data and its accumulators
 struct RowDF {
   int pi;
@@ -117,6 +160,7 @@ struct RowDF {
   float xf, yf, zf, vxf, vyf, vzf, lam, sig;   // kick 1: FP32 prefilter copies
   int gid;                 // kick 2: encounter group
   df acc[3];               // carried across the macro-tile's column blocks
+  float lost;              // sum of s GRID_TERM
 };
 
 // a column body in shared memory: {x: a b c, y: a} {y: b c, z: a b} {z: c, G m: h l, group}
@@ -125,7 +169,8 @@ struct ColDF {
 };
 
 template <int MODE>
-__device__ __forceinline__ void row_load_df(const Dev &D, const TileCtx &c, const int *E, int I, int lane, RowDF &r) {
+__device__ __forceinline__ void row_load_df(const Dev &D, const TileCtx &c, const int *E, const Units &u, int I, int lane,
+                                            RowDF &r) {
   r.pi = I * 32 + lane;
   const int li = r.pi - c.off;
   r.live = li < c.n && D.alive[r.pi];
@@ -133,10 +178,11 @@ __device__ __forceinline__ void row_load_df(const Dev &D, const TileCtx &c, cons
   const double p[3] = {D.x[r.pi], D.y[r.pi], D.z[r.pi]};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    on_grid(r.live ? p[k] : 0.0, E[k], c.kex, r.x[k][0], r.x[k][1], r.x[k][2]);
+    on_grid(r.live ? p[k] : 0.0, E[k], u.kex, r.x[k][0], r.x[k][1], r.x[k][2]);
     r.acc[k] = mk(0.0f, 0.0f);
   }
-  r.ngm = neg(split(scale2(D.gm[r.pi], -c.keg)));
+  r.lost = 0.0f;
+  r.ngm = neg(split(scale2(D.gm[r.pi], -u.keg)));
   r.xf = r.yf = r.zf = r.vxf = r.vyf = r.vzf = r.lam = r.sig = 0.f;
   r.gid = -1;
   if (MODE == 1) {
@@ -158,11 +204,12 @@ __device__ __forceinline__ df weighted(df s, double w) { return w == 0.0 ? mk(0.
 template <int MODE>
 __device__ __forceinline__ void tile_steps_df(const Dev &D, const TileCtx &c, int sys, RowDF &r, int I, int J, int lane,
                                               int t0, int t1, const ColDF *col, const float4 (*cf)[2],
-                                              unsigned mlive, unsigned mmass, float2 (*out)[32]) {
+                                              unsigned mlive, unsigned mmass, float2 (*out)[32], float *out_lost) {
   const bool diag = I == J;
   const int o = diag ? 1 : 0;
   const float tauf = __double2float_ru(c.dt);
   df ca[3] = {mk(0.0f, 0.0f), mk(0.0f, 0.0f), mk(0.0f, 0.0f)};
+  float lost = 0.0f;
 #pragma unroll 1
   for (int t = t0; t < t1; ++t) {
     const int cj = (lane + t + o) & 31;
@@ -231,8 +278,11 @@ __device__ __forceinline__ void tile_steps_df(const Dev &D, const TileCtx &c, in
       accumulate(r.acc[k], mul(sj, d[k]));
       accumulate(ca[k], mul(si, d[k]));
     }
+    r.lost = fmaf(fabsf(sj.h), GRID_TERM, r.lost);
+    lost = fmaf(fabsf(si.h), GRID_TERM, lost);
     if (t + 1 < t1) {
       const int src = (lane + 1) & 31;
+      lost = __shfl_sync(FULL, lost, src);
 #pragma unroll
       for (int k = 0; k < 3; ++k) ca[k] = mk(__shfl_sync(FULL, ca[k].h, src), __shfl_sync(FULL, ca[k].l, src));
     }
@@ -243,6 +293,63 @@ __device__ __forceinline__ void tile_steps_df(const Dev &D, const TileCtx &c, in
     const df q = t1 > t0 ? renorm(ca[k]) : ca[k];
     out[k][last] = make_float2(q.h, q.l);
   }
+  out_lost[last] = lost;
+}
+
+// The macro-tile again in FP64 (its encounters are in the pair list already): the same warps, quarters and
+// order, sums into the same slots.  For the rare macro-tile, so bodies are read where they lie.
+template <int MODE>
+static __device__ __noinline__ void macro_general(const Dev &D, const int4 mt, const ColDF (*col)[32], const float4 (*cf)[32][2],
+                                                  const unsigned *mlive, const unsigned *mmass, double (*rowbuf)[3][32],
+                                                  double (*colbuf)[MC][3][32]) {
+  const TileCtx c = load_ctx(&D.disks[mt.x]);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ws = w >> 2, I = mt.y + (w & 3), pi = I * 32 + lane;
+  const bool has_row = I < mt.w;
+  const int q = has_row ? pi : c.off, li = pi - c.off;
+  const bool live = has_row && li < c.n && D.alive[q], row = live && li < c.nm;
+  const double x = D.x[q], y = D.y[q], z = D.z[q], ngm = -D.gm[q];
+  const float tauf = __double2float_ru(c.dt);
+  double ra[3] = {0.0, 0.0, 0.0};
+  for (int k = 0; k < MC; ++k) {
+    const int J = mt.z + k;
+    const bool diag = I == J, any = has_row && J < mt.w && J >= I;
+    const int len = any ? (diag ? 4 : 8) : 0, o = diag ? 1 : 0;
+    double ca[3] = {0.0, 0.0, 0.0};
+    for (int t = len * ws; t < len * ws + len; ++t) {
+      const int cj = (lane + t + o) & 31, jid = J * 32 + cj;
+      const bool jl = (mlive[k] >> cj) & 1u, jm = (mmass[k] >> cj) & 1u;
+      bool valid = diag ? (jid > pi ? (row && jl) : (live && jm)) : (row && jl);
+      if (diag && t == 15 && lane >= 16) valid = false;
+      const double dx = D.x[jid] - x, dy = D.y[jid] - y, dz = D.z[jid] - z;
+      const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+      const double ri = rsqrt_fp64(r2), r3 = ri * ri * ri;
+      double wt = 1.0;
+      if (valid) {
+        const int lo = min(pi, jid), hi = max(pi, jid);
+        if (MODE == 1) {
+          const float4 fa = cf[k][cj][0], fb = cf[k][cj][1];
+          const float dxf = fa.x - D.xf[pi], dyf = fa.y - D.yf[pi], dzf = fa.z - D.zf[pi];
+          const float r2f = fmaf(dzf, dzf, fmaf(dyf, dyf, dxf * dxf));
+          const float dvxf = fa.w - D.vxf[pi], dvyf = fb.x - D.vyf[pi], dvzf = fb.y - D.vzf[pi];
+          const float vmag = sqrtf(fmaf(dvzf, dvzf, fmaf(dvyf, dvyf, dvxf * dvxf)));
+          const float Bf = fmaf(tauf, vmag, D.lamf[pi] + fb.z) * 1.0000039f + 1.9073486e-6f * (D.sigf[pi] + fb.w);
+          if (!(r2f > Bf * Bf)) wt = flagged_weight(D, c, lo, hi);
+        } else if (D.gid[pi] >= 0 && D.gid[pi] == __float_as_int(col[k][cj].q[2].w) && group_has_pair(D, D.gid[pi], lo, hi)) {
+          wt = g0_weight(c, __dmul_rn(c.lam, __dadd_rn(D.rh[lo], D.rh[hi])), sqrt(r2));
+        }
+      }
+      const double sj = valid && wt != 0.0 ? D.gm[jid] * r3 * wt : 0.0, si = valid && wt != 0.0 ? ngm * r3 * wt : 0.0;
+      ra[0] = fma(sj, dx, ra[0]); ra[1] = fma(sj, dy, ra[1]); ra[2] = fma(sj, dz, ra[2]);
+      ca[0] = fma(si, dx, ca[0]); ca[1] = fma(si, dy, ca[1]); ca[2] = fma(si, dz, ca[2]);
+      if (t + 1 < len * ws + len) {
+        const int src = (lane + 1) & 31;
+        for (int e = 0; e < 3; ++e) ca[e] = __shfl_sync(FULL, ca[e], src);
+      }
+    }
+    const int last = (lane + len * ws + len - 1 + o) & 31;
+    for (int e = 0; e < 3; ++e) colbuf[w][k][e][len ? last : lane] = ca[e];
+  }
+  for (int e = 0; e < 3; ++e) rowbuf[w][e][lane] = ra[e];
 }
 
 // Mixed precision (FP32 pair path): the relative displacement is formed from the two-float split
@@ -410,21 +517,22 @@ __device__ __forceinline__ void tile_sweep_mixed(const Dev &D, const TileCtx &c,
 // each of its tiles, so that a system of a few blocks (one macro-tile per 128 x 64 bodies) still fills
 // the SM it runs on: the 1,000-body disk has 80 macro-tiles for 152 SMs.
 template <int MODE>
-__global__ void __launch_bounds__(512) k_trap_df(Dev D) {
+__global__ void __launch_bounds__(512) k_trap_df(const __grid_constant__ Dev D) {
   __shared__ ColDF col[MC][32];
   __shared__ float4 cf[MC][32][2];              // kick 1: xf, yf, zf, vxf | vyf, vzf, lambda, sigma
   __shared__ float2 rowbuf[16][3][32];          // [warp][component][lane]
   __shared__ float2 colbuf[16][MC][3][32];
-  __shared__ int s_max[3];
+  __shared__ float rowlost[16][32], collost[16][MC][32];
+  __shared__ int s_max[4], s_min;               // high words of the largest |x|, |y|, |z|, G m; smallest G m > 0
+  __shared__ int s_v[4 + MC][32];               // of each body's largest |v| component; -1: no live body
   __shared__ unsigned s_live[MC], s_mass[MC];
   __shared__ int s_item;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wr = w & 3, ws = w >> 2;
   const int nmac = D.ntiles_total;
   const int S = D.seg_len;
   int *counter = &D.work[MODE - 1];
-  float2 *part = reinterpret_cast<float2 *>(D.part);
-  if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-  if (threadIdx.x < 3) s_max[threadIdx.x] = 0;
+  if (threadIdx.x == 0) { s_item = atomicAdd(counter, 1); s_min = 0x7FFFFFFF; }
+  if (threadIdx.x < 4) s_max[threadIdx.x] = 0;
   __syncthreads();
   int m0 = s_item * S;
   while (m0 < nmac) {
@@ -432,21 +540,27 @@ __global__ void __launch_bounds__(512) k_trap_df(Dev D) {
     for (int m = m0; m < m1; ++m) {
       const int4 mt = D.tiles[m];
       const TileCtx c = load_ctx(&D.disks[mt.x]);
-      // the grids: largest |x| of the macro-tile's live bodies, component by component
+      // the units and grids: largest |x|, component by component, and G m of the macro-tile's live bodies
       if (w < 4 + MC) {
         const int b = w < 4 ? mt.y + w : mt.z + (w - 4);
         const int p = b * 32 + lane;
         const bool in = b < mt.w && p - c.off < c.n && D.alive[p];
-        const double *xs[3] = {D.x, D.y, D.z};
+        const double *xs[4] = {D.x, D.y, D.z, D.gm};
+        auto hi = [&](const double *a) { return in ? __double2hiint(a[p]) & 0x7FFFFFFF : 0; };
+        s_v[w][lane] = in ? max(hi(D.vx), max(hi(D.vy), hi(D.vz))) : -1;
+        int h = 0;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const unsigned hi = in ? (unsigned)__double2hiint(xs[k][p]) & 0x7FFFFFFFu : 0u;
-          const unsigned top = __reduce_max_sync(FULL, hi);
-          if (lane == 0) atomicMax(&s_max[k], (int)top);
+        for (int k = 0; k < 4; ++k) {
+          h = hi(xs[k]);
+          const int top = __reduce_max_sync(FULL, h);
+          if (lane == 0) atomicMax(&s_max[k], top);
         }
+        const int low = __reduce_min_sync(FULL, h ? h : 0x7FFFFFFF);
+        if (lane == 0) atomicMin(&s_min, low);
       }
       __syncthreads();
-      const int E[3] = {grid_exp(s_max[0], c.kex), grid_exp(s_max[1], c.kex), grid_exp(s_max[2], c.kex)};
+      const Units u = units_of(s_max[0], s_max[1], s_max[2], s_max[3], s_min);
+      const int E[3] = {grid_exp(s_max[0], u.kex), grid_exp(s_max[1], u.kex), grid_exp(s_max[2], u.kex)};
       if (w >= 16 - MC) {                       // the last warps stage the column blocks
         const int k = w - (16 - MC), b = mt.z + k, j = b * 32 + lane;
         const bool in = b < mt.w, live = in && j - c.off < c.n && D.alive[j];
@@ -456,8 +570,8 @@ __global__ void __launch_bounds__(512) k_trap_df(Dev D) {
           float g[3][3];
           const double p[3] = {D.x[j], D.y[j], D.z[j]};
 #pragma unroll
-          for (int q = 0; q < 3; ++q) on_grid(live ? p[q] : 0.0, E[q], c.kex, g[q][0], g[q][1], g[q][2]);
-          const df gm = split(scale2(D.gm[j], -c.keg));
+          for (int q = 0; q < 3; ++q) on_grid(live ? p[q] : 0.0, E[q], u.kex, g[q][0], g[q][1], g[q][2]);
+          const df gm = split(scale2(D.gm[j], -u.keg));
           col[k][lane].q[0] = make_float4(g[0][0], g[0][1], g[0][2], g[1][0]);
           col[k][lane].q[1] = make_float4(g[1][1], g[1][2], g[2][0], g[2][1]);
           col[k][lane].q[2] = make_float4(g[2][2], gm.h, gm.l, __int_as_float(MODE == 2 ? D.gid[j] : -1));
@@ -470,7 +584,7 @@ __global__ void __launch_bounds__(512) k_trap_df(Dev D) {
       const int I = mt.y + wr;
       const bool has_row = I < mt.w;
       RowDF r;
-      if (has_row) row_load_df<MODE>(D, c, E, I, lane, r);
+      if (has_row) row_load_df<MODE>(D, c, E, u, I, lane, r);
       __syncthreads();
 #pragma unroll 1
       for (int k = 0; k < MC; ++k) {
@@ -478,10 +592,11 @@ __global__ void __launch_bounds__(512) k_trap_df(Dev D) {
         if (has_row && J < mt.w && J >= I) {
           const int q = I == J ? 4 : 8;         // a quarter of 16 or 32 steps
           tile_steps_df<MODE>(D, c, mt.x, r, I, J, lane, q * ws, q * ws + q, col[k], cf[k], s_live[k], s_mass[k],
-                              colbuf[w][k]);
+                              colbuf[w][k], collost[w][k]);
         } else {
 #pragma unroll
           for (int q = 0; q < 3; ++q) colbuf[w][k][q][lane] = make_float2(0.0f, 0.0f);
+          collost[w][k][lane] = 0.0f;
         }
       }
 #pragma unroll
@@ -489,12 +604,30 @@ __global__ void __launch_bounds__(512) k_trap_df(Dev D) {
         const df a = has_row ? renorm(r.acc[q]) : mk(0.0f, 0.0f);
         rowbuf[w][q][lane] = make_float2(a.h, a.l);
       }
+      rowlost[w][lane] = has_row ? r.lost : 0.0f;
       // the next item is taken while the sums are formed (everyone has read s_item)
-      if (threadIdx.x < 3) s_max[threadIdx.x] = 0;
-      if (m + 1 == m1 && threadIdx.x == 0) s_item = atomicAdd(counter, 1);
+      if (threadIdx.x < 4) s_max[threadIdx.x] = 0;
+      if (threadIdx.x == 0) {
+        s_min = 0x7FFFFFFF;
+        if (m + 1 == m1) s_item = atomicAdd(counter, 1);
+      }
       __syncthreads();
+      double *part = D.part + (size_t)m * SYM_MACRO_PART;
+      bool general = !u.fits;
       for (int i = threadIdx.x; i < SYM_MACRO_PART; i += 512) {     // [4 rows, MC columns][component][lane]
         const int blk = i / 96, q = (i / 32) % 3, l = i & 31;
+        if (q == 0 && s_v[blk][l] >= 0) {
+          float lost = 0.0f;
+          if (blk < 4) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) lost += rowlost[4 * v + blk][l];
+          } else {
+#pragma unroll
+            for (int v = 0; v < 16; ++v) lost += collost[v][blk - 4][l];
+          }
+          const int ng = (mt.w - (c.off >> 5) + MC - 1) / MC;       // at most ng + 1 sums for a body
+          if (!(lost <= error_room(s_v[blk][l], c.dt, u, ng + 1))) general = true;
+        }
         df a = mk(0.0f, 0.0f);
         if (blk < 4) {
 #pragma unroll
@@ -503,10 +636,21 @@ __global__ void __launch_bounds__(512) k_trap_df(Dev D) {
 #pragma unroll 4
           for (int v = 0; v < 16; ++v) accumulate(a, ld2(colbuf[v][blk - 4][q][l]));
         }
-        a = renorm(a);
-        part[(size_t)m * SYM_MACRO_PART + i] = make_float2(a.h, a.l);
+        part[i] = kick_value(a, u.keg - 2 * u.kex);
       }
-      __syncthreads();                          // the buffers are free
+      if (__syncthreads_or(general)) {          // (and the buffers are free)
+        auto rows = reinterpret_cast<double (*)[3][32]>(rowbuf);
+        auto cols = reinterpret_cast<double (*)[MC][3][32]>(colbuf);
+        macro_general<MODE>(D, mt, col, cf, s_live, s_mass, rows, cols);
+        __syncthreads();
+        for (int i = threadIdx.x; i < SYM_MACRO_PART; i += 512) {
+          const int blk = i / 96, q = (i / 32) % 3, l = i & 31;
+          double a = 0.0;
+          for (int v = blk < 4 ? blk : 0; v < 16; v += blk < 4 ? 4 : 1) a += blk < 4 ? rows[v][q][l] : cols[v][blk - 4][q][l];
+          part[i] = a;
+        }
+        __syncthreads();
+      }
     }
     m0 = s_item * S;
   }
@@ -658,14 +802,47 @@ __device__ __forceinline__ double field_check(const Dev &D, const TileCtx &c, in
   return g0_weight(c, R0, __dsqrt_rn(er2));
 }
 
-// FP64 systems, in double-float as the tiles: one CTA per field block, its four warps each taking every
-// fourth chunk of 32 massive bodies; the four sums are added in warp order.
+// FP64 systems, in double-float as the tiles, with units of each chunk's own: one CTA per field block, its
+// four warps each taking every fourth chunk of 32 massive bodies; a chunk's sum joins the warp's in FP64, the
+// four sums are added in warp order.  A chunk where a particle's error may exceed its share of the rounding
+// of v (as in the tiles) is taken again in FP64, bodies read where they lie:
 template <int MODE>
-__global__ void __launch_bounds__(128) k_field_df(Dev D) {
+static __device__ __noinline__ double3 field_chunk_general(const Dev &D, int sys, int p, bool live, int c0, const float4 (*cf)[2]) {
+  const TileCtx c = load_ctx(&D.disks[sys]);
+  const float tauf = __double2float_ru(c.dt);
+  const double x = D.x[p], y = D.y[p], z = D.z[p];
+  const int cnt = min(32, c.nm - c0);
+  double3 a = make_double3(0.0, 0.0, 0.0);
+  for (int s = 0; s < cnt; ++s) {
+    const int id = c.off + c0 + s;
+    const bool valid = live && D.alive[id];
+    const double dx = D.x[id] - x, dy = D.y[id] - y, dz = D.z[id] - z;
+    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+    const double ri = rsqrt_fp64(r2);
+    double wt = 1.0;
+    if (valid && MODE == 1) {
+      const float4 fa = cf[s][0], fq = cf[s][1];
+      const float dxf = fa.x - D.xf[p], dyf = fa.y - D.yf[p], dzf = fa.z - D.zf[p];
+      const float r2f = fmaf(dzf, dzf, fmaf(dyf, dyf, dxf * dxf));
+      const float dvxf = fa.w - D.vxf[p], dvyf = fq.x - D.vyf[p], dvzf = fq.y - D.vzf[p];
+      const float vmag = sqrtf(fmaf(dvzf, dvzf, fmaf(dvyf, dvyf, dvxf * dvxf)));
+      const float Bf = fmaf(tauf, vmag, fq.z + D.lamf[p]) * 1.0000039f + 1.9073486e-6f * (fq.w + D.sigf[p]);
+      if (!(r2f > Bf * Bf)) wt = flagged_weight(D, c, id, p);
+    } else if (valid && D.gid[p] >= 0 && D.gid[p] == D.gid[id] && group_has_pair(D, D.gid[p], id, p)) {
+      wt = g0_weight(c, __dmul_rn(c.lam, __dadd_rn(D.rh[id], D.rh[p])), sqrt(r2));
+    }
+    const double sp = valid && wt != 0.0 ? D.gm[id] * (ri * ri * ri) * wt : 0.0;
+    a.x = fma(sp, dx, a.x); a.y = fma(sp, dy, a.y); a.z = fma(sp, dz, a.z);
+  }
+  return a;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(128) k_field_df(const __grid_constant__ Dev D) {
   __shared__ ColDF col[4][32];
   __shared__ float4 cf[4][32][2];
   __shared__ int sid[4][32];
-  __shared__ float2 sums[4][3][32];
+  __shared__ double sums[4][3][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int2 fb = D.fblk[blockIdx.x];            // {system, global block}
   const TileCtx c = load_ctx(&D.disks[fb.x]);
@@ -677,6 +854,8 @@ __global__ void __launch_bounds__(128) k_field_df(Dev D) {
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     top[k] = (int)__reduce_max_sync(FULL, live ? (unsigned)__double2hiint(xp[k]) & 0x7FFFFFFFu : 0u);
+  auto hi = [](double a) { return __double2hiint(a) & 0x7FFFFFFF; };
+  const int hv = max(hi(D.vx[p]), max(hi(D.vy[p]), hi(D.vz[p])));
   const float xfp = D.xf[p], yfp = D.yf[p], zfp = D.zf[p];
   float vxfp = 0.f, vyfp = 0.f, vzfp = 0.f, lamp = 0.f, sigp = 0.f;
   int gidp = -1;
@@ -686,21 +865,27 @@ __global__ void __launch_bounds__(128) k_field_df(Dev D) {
     gidp = D.gid[p];
   }
   const float tauf = __double2float_ru(c.dt);
-  df acc[3] = {mk(0.0f, 0.0f), mk(0.0f, 0.0f), mk(0.0f, 0.0f)};
+  double tot[3] = {0.0, 0.0, 0.0};
   for (int c0 = 32 * w; c0 < c.nm; c0 += 128) {
     const int li = c0 + lane, j = c.off + li;
     const bool ok = li < c.nm && D.alive[j];
     const int jq = ok ? j : c.off;                // a valid address for the loads below
     const double xj[3] = {D.x[jq], D.y[jq], D.z[jq]};
     float g[3][3], gp[3][3];
+    int t[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t[k] = max(top[k], __reduce_max_sync(FULL, ok ? hi(xj[k]) : 0));
+    const int hg = ok ? hi(D.gm[jq]) : 0;
+    const Units u = units_of(t[0], t[1], t[2], __reduce_max_sync(FULL, hg), __reduce_min_sync(FULL, hg ? hg : 0x7FFFFFFF));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const int t = (int)__reduce_max_sync(FULL, ok ? (unsigned)__double2hiint(xj[k]) & 0x7FFFFFFFu : 0u);
-      const int E = grid_exp(max(t, top[k]), c.kex);
-      on_grid(ok ? xj[k] : 0.0, E, c.kex, g[k][0], g[k][1], g[k][2]);
-      on_grid(live ? xp[k] : 0.0, E, c.kex, gp[k][0], gp[k][1], gp[k][2]);
+      const int E = grid_exp(t[k], u.kex);
+      on_grid(ok ? xj[k] : 0.0, E, u.kex, g[k][0], g[k][1], g[k][2]);
+      on_grid(live ? xp[k] : 0.0, E, u.kex, gp[k][0], gp[k][1], gp[k][2]);
     }
-    const df gm = split(scale2(D.gm[jq], -c.keg));
+    const df gm = split(scale2(D.gm[jq], -u.keg));
+    df acc[3] = {mk(0.0f, 0.0f), mk(0.0f, 0.0f), mk(0.0f, 0.0f)};
+    float lost = 0.0f;
     __syncwarp();
     col[w][lane].q[0] = make_float4(g[0][0], g[0][1], g[0][2], g[1][0]);
     col[w][lane].q[1] = make_float4(g[1][1], g[1][2], g[2][0], g[2][1]);
@@ -747,20 +932,24 @@ __global__ void __launch_bounds__(128) k_field_df(Dev D) {
       sp.l = valid ? sp.l : 0.0f;
 #pragma unroll
       for (int k = 0; k < 3; ++k) accumulate(acc[k], mul(sp, d[k]));
+      lost = fmaf(fabsf(sp.h), GRID_TERM, lost);
+    }
+    const bool good = u.fits && (!live || lost <= error_room(hv, c.dt, u, (c.nm + 31) / 32));
+    if (__all_sync(FULL, good)) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) tot[k] += kick_value(acc[k], u.keg - 2 * u.kex);
+    } else {
+      const double3 a = field_chunk_general<MODE>(D, fb.x, p, live, c0, cf[w]);
+      tot[0] += a.x; tot[1] += a.y; tot[2] += a.z;
     }
   }
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const df a = renorm(acc[k]);
-    sums[w][k][lane] = make_float2(a.h, a.l);
-  }
+  for (int k = 0; k < 3; ++k) sums[w][k][lane] = tot[k];
   __syncthreads();
   if (w < 3 && live) {                           // warp w adds component w
-    df a = mk(0.0f, 0.0f);
-#pragma unroll
-    for (int v = 0; v < 4; ++v) accumulate(a, ld2(sums[v][w][lane]));
+    const double a = (sums[0][w][lane] + sums[1][w][lane]) + (sums[2][w][lane] + sums[3][w][lane]);
     double *vel = w == 0 ? D.vx : (w == 1 ? D.vy : D.vz);
-    vel[p] = __dadd_rn(vel[p], __dmul_rn(0.5 * c.dt, kick_value(a, c.keg - 2 * c.kex)));
+    vel[p] = __dadd_rn(vel[p], __dmul_rn(0.5 * c.dt, a));
   }
 }
 
