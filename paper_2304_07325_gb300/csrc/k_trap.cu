@@ -120,13 +120,15 @@ __device__ __forceinline__ void accumulate(df &sum, df t) {
 // ---- how far the double-float form may go
 // Positions are scaled by 2^-kex and G m by 2^-keg, the largest of the macro-tile (of the field chunk), so
 // neither what lies elsewhere in the system nor how far it has spread since set-up matters.  What is lost:
-// the grid moves a separation by up to sqrt(3) 2^-61, which changes a pair's force s d (s = G m / r^3) by
-// up to 4 sqrt(3) 2^-61 s < 2^-58 s.  Every body's sum of s GRID_TERM 2^-46 is kept beside its force and
-// the macro-tile is taken again in FP64 (macro_general) when, times tau/2, it may exceed 2^-54 |v| of a
-// body -- half of what the rounding of v loses anyway -- or when a force left the FP32 range.  So a body far
-// from the rest (ejected, or parked) costs the macro-tiles it is in time and not accuracy: for pairs 0.05 AU
-// apart in a disk of 10 AU the double-float force is off by 2e-16 of itself, and with a body of the
-// macro-tile at 1e8 AU by 1.5e-9.
+// the arithmetic leaves an error of about 2^-46 of a pair's force s d, s = G m / r^3, and the grid moves a
+// separation by up to sqrt(3) 2^-61, which changes the force by up to 4 sqrt(3) 2^-61 s < 2^-58 s.  Every
+// body's sum of s (r + GRID_TERM) is kept beside its force, and the macro-tile is taken again in FP64
+// (macro_general) when 2^-46 of it, times tau/2, may exceed 2^-54 |v| of a body -- half of what the rounding
+// of v loses anyway -- or when a force left the FP32 range.  So kicks above 2^-8 |v| (a body of 1e-3 m0 five
+// mutual Hill radii away, tau a tenth of the period) keep FP64's digits, and a body far from the rest
+// (ejected, or parked) costs the macro-tiles it is in time and not accuracy: for pairs 0.05 AU apart in a
+// disk of 10 AU the double-float force is off by 2e-16 of itself, and with a body of the macro-tile at
+// 1e8 AU by 1.5e-9.
 #define GRID_TERM 2.4414062e-4f          // 2^-12
 struct Units {
   int kex, keg;
@@ -142,7 +144,7 @@ __device__ __forceinline__ Units units_of(int hx, int hy, int hz, int gmax, int 
   u.fits = abs(u.kex) <= 250 && abs(u.keg) <= 250 && (gmax == 0 || top_exp(gmin) >= u.keg - 80);
   return u;
 }
-// Largest sum of s GRID_TERM (scaled) allowed for a body: 2^-8 |v| / (tau/2) over the square root of the
+// Largest sum of s (r + GRID_TERM) (scaled) allowed for a body: 2^-8 |v| / (tau/2) over the square root of the
 // number of such sums (their errors are independent), rounded down to a power of two.  hv: high word of
 // the body's largest |v| component.
 __device__ __forceinline__ float error_room(int hv, double dt, const Units &u, int nsum) {
@@ -160,7 +162,7 @@ struct RowDF {
   float xf, yf, zf, vxf, vyf, vzf, lam, sig;   // kick 1: FP32 prefilter copies
   int gid;                 // kick 2: encounter group
   df acc[3];               // carried across the macro-tile's column blocks
-  float lost;              // sum of s GRID_TERM
+  float lost;              // sum of s (r + GRID_TERM)
 };
 
 // a column body in shared memory: {x: a b c, y: a} {y: b c, z: a b} {z: c, G m: h l, group}
@@ -226,7 +228,10 @@ __device__ __forceinline__ void tile_steps_df(const Dev &D, const TileCtx &c, in
     const df d[3] = {separation(q0.x, q0.y, q0.z, r.x[0][0], r.x[0][1], r.x[0][2]),
                      separation(q0.w, q1.x, q1.y, r.x[1][0], r.x[1][1], r.x[1][2]),
                      separation(q1.z, q1.w, q2.x, r.x[2][0], r.x[2][1], r.x[2][2])};
-    const df r3 = inverse_cube(root(norm2(d)));
+    const df r2 = norm2(d);
+    const df_root rt = root(r2);
+    const float reach = fminf(fmaf(r2.h, rt.y, GRID_TERM), 8.0f);     // (8 where r = 0: a pair left out)
+    const df r3 = inverse_cube(rt);
     df sj = mul(mk(q2.y, q2.z), r3);
     df si = mul(r.ngm, r3);             // the column side's -G m_i / r^3
     if (MODE == 1) {
@@ -278,8 +283,8 @@ __device__ __forceinline__ void tile_steps_df(const Dev &D, const TileCtx &c, in
       accumulate(r.acc[k], mul(sj, d[k]));
       accumulate(ca[k], mul(si, d[k]));
     }
-    r.lost = fmaf(fabsf(sj.h), GRID_TERM, r.lost);
-    lost = fmaf(fabsf(si.h), GRID_TERM, lost);
+    r.lost = fmaf(fabsf(sj.h), reach, r.lost);
+    lost = fmaf(fabsf(si.h), reach, lost);
     if (t + 1 < t1) {
       const int src = (lane + 1) & 31;
       lost = __shfl_sync(FULL, lost, src);
@@ -905,7 +910,9 @@ __global__ void __launch_bounds__(128) k_field_df(const __grid_constant__ Dev D)
       const df d[3] = {separation(q0.x, q0.y, q0.z, gp[0][0], gp[0][1], gp[0][2]),
                        separation(q0.w, q1.x, q1.y, gp[1][0], gp[1][1], gp[1][2]),
                        separation(q1.z, q1.w, q2.x, gp[2][0], gp[2][1], gp[2][2])};
-      df sp = mul(mk(q2.y, q2.z), inverse_cube(root(norm2(d))));
+      const df r2 = norm2(d);
+      const df_root rt = root(r2);
+      df sp = mul(mk(q2.y, q2.z), inverse_cube(rt));
       if (MODE == 1) {
         const float4 fa = cf[w][s][0], fq = cf[w][s][1];
         const float dxf = fa.x - xfp, dyf = fa.y - yfp, dzf = fa.z - zfp;
@@ -932,7 +939,7 @@ __global__ void __launch_bounds__(128) k_field_df(const __grid_constant__ Dev D)
       sp.l = valid ? sp.l : 0.0f;
 #pragma unroll
       for (int k = 0; k < 3; ++k) accumulate(acc[k], mul(sp, d[k]));
-      lost = fmaf(fabsf(sp.h), GRID_TERM, lost);
+      lost = fmaf(fabsf(sp.h), fminf(fmaf(r2.h, rt.y, GRID_TERM), 8.0f), lost);
     }
     const bool good = u.fits && (!live || lost <= error_room(hv, c.dt, u, (c.nm + 31) / 32));
     if (__all_sync(FULL, good)) {
