@@ -108,7 +108,8 @@ struct symba_pool {
   int rec_bpsm = 1;
   int group_order = 0;
   bool any_discard = false;   // some system has a removal distance: the step runs k_discard
-  // held while work that uses the recursion's scratch is enqueued: a step, or a read that stages in it
+  // held while work that uses the recursion's scratch is enqueued: a step, the autotuner's trial steps (until
+  // the state is put back), or a read that stages in it
   std::mutex scratch;
   std::unique_ptr<char[]> host;   // a small read's arrays on the host (READ_PACK bytes)
 };
@@ -735,6 +736,8 @@ int copy_spans(const std::vector<Span> &v, char *buf, bool save, cudaStream_t s)
 int pool_autotune(symba_pool *P, int reps, symba_tune_result *out) {
   if (reps < 1) return SYMBA_E_INVAL;
   CK(cudaSetDevice(P->device));
+  // (a read of another thread waits: it would find a trial step's forces where it stages, or a trial state)
+  std::lock_guard<std::mutex> lock(P->scratch);
   symba_tune_result r;
   memset(&r, 0, sizeof(r));
   get_schedule(P, &r.chosen);
