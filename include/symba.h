@@ -168,8 +168,8 @@ int symba_get_stats(symba_ctx *c, symba_stats *s);
  * summed device time of each phase in milliseconds to phase_ms[0..SYMBA_NPHASES-1] (host):
  * 0 sun drift + step prologue, 1 kick 1 with the fused encounter check, 2 kick-1 reduction,
  * 3 grouping, 4 Kepler drift, 5 group recursion, 6 kick 2, 7 kick-2 reduction,
- * 8 total momentum with the closing sun drift, 9 nothing since then (zero; kept in the
- * layout).  Returns the sticky status like symba_sync. */
+ * 8 total momentum, 9 closing sun drift (a step of small systems takes these two in one kernel,
+ * with the same result).  Returns the sticky status like symba_sync. */
 #define SYMBA_NPHASES 10
 int symba_profile_step(symba_ctx *c, int nsteps, double *phase_ms);
 

@@ -315,8 +315,9 @@ int pool_profile(symba_pool *P, int nsteps, double *phase_ms) {
     launch_reduce(D, np, P->precision, s);
     if (P->any_discard) launch_discard(D, np, s);
     cudaEventRecord(ev[8], s);
-    launch_momentum(D, P->ndisks, np, P->n_max, true, s);
-    cudaEventRecord(ev[9], s);             // (the closing drift is launched with the momentum)
+    launch_momentum(D, P->ndisks, np, P->n_max, false, s);
+    cudaEventRecord(ev[9], s);
+    launch_close(D, np, s);                // (by itself also where a step's momentum kernel drifts: same bits)
     cudaEventRecord(ev[10], s);
     if (cudaEventSynchronize(ev[10]) != cudaSuccess) { rc = SYMBA_E_CUDA; break; }
     for (int k = 0; k < SYMBA_NPHASES; ++k) {

@@ -488,6 +488,8 @@ void launch_init_state(const Dev &D, int d, int n, const double *xh, const doubl
                        cudaStream_t s);
 // total momentum of every system (n_max: bodies of the largest); drift: and the closing sun drift
 void launch_momentum(const Dev &D, int ndisks, long long npart, int n_max, bool drift, cudaStream_t s);
+// closing sun drift by itself (phase timing)
+void launch_close(const Dev &D, long long npart, cudaStream_t s);
 // opening sun drift of a step, with the reset of the per-step counters
 void launch_open(const Dev &D, long long npart, int ndisks, cudaStream_t s);
 void launch_trap(const Dev &D, const LaunchCfg &L, int mode, int precision, cudaStream_t s);

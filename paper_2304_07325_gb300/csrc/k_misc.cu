@@ -307,6 +307,10 @@ void launch_open(const Dev &D, long long npart, int ndisks, cudaStream_t s) {
   k_sundrift<true><<<sundrift_blocks(npart), 256, 0, s>>>(D, npart, ndisks);
 }
 
+void launch_close(const Dev &D, long long npart, cudaStream_t s) {
+  if (npart > 0) k_sundrift<false><<<sundrift_blocks(npart), 256, 0, s>>>(D, npart, 0);
+}
+
 void launch_momentum(const Dev &D, int ndisks, long long npart, int n_max, bool drift, cudaStream_t s) {
   if (ndisks <= 0) return;
   if (n_max <= MOM_ONE_MAX) {
@@ -315,7 +319,7 @@ void launch_momentum(const Dev &D, int ndisks, long long npart, int n_max, bool 
   }
   k_momentum_acc<<<dim3(MOM_CTAS, ndisks), 256, 0, s>>>(D);
   k_momentum_round<<<ndisks, 96, 0, s>>>(D);
-  if (drift && npart > 0) k_sundrift<false><<<sundrift_blocks(npart), 256, 0, s>>>(D, npart, ndisks);
+  if (drift) launch_close(D, npart, s);
 }
 
 // --------------------------------------------------------------------------------------------
