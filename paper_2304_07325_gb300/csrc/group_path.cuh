@@ -17,19 +17,26 @@
 // two binaries in a group of 42 bodies 117 -> 45; 260 disks of 500 to 4,000 bodies 4.3 times as fast
 // (geometric mean, with the single-pair path's share).
 
-// the group's units, |x| ~ 2^ea and |v| ~ 2^eb, and whether its quantities are normal FP32 numbers in
-// them, with room for their products
+// The group's units, |x| ~ 2^ea and |v| ~ 2^eb, and whether its quantities are normal FP32 numbers in them,
+// with room for their products, at every level down to max_depth (h_k falls by M per level, R_k by the shell
+// ratio).  At the deepest:
+//   R_{k+1}: the force of level k is used from there on, and r^-3, times G m, stays below 2^125;
+//   G m h/2: not below 2^-100, from where on its low part would be lost;
+//   h: not below 2^-70, so that h times what FP64 still adds to v (2^-53) is a normal number.
+// (The sun's mu h^2 may leave the range: what it then moves v by is below 2^-63 per sub-step.)
 struct GroupScale {
   int ea, eb;
   bool fits;
 };
 __device__ GroupScale group_scale(const GView &S, const GroupCtx &C, int lane) {
-  unsigned mx = 0u, mv = 0u, mg = 0u;
+  auto hi = [](double t) { return (unsigned)__double2hiint(t) & 0x7FFFFFFFu; };
+  auto top = [&](double t) { return (int)(hi(t) >> 20) - 1023; };
+  unsigned mx = 0u, mv = 0u, mg = 0u, lg = 0x7FFFFFFFu;
   for (int a = lane; a < C.mcnt; a += 32) {
-    auto hi = [](double t) { return (unsigned)__double2hiint(t) & 0x7FFFFFFFu; };
     mx = max(mx, max(hi(S.x[a]), max(hi(S.y[a]), hi(S.z[a]))));
     mv = max(mv, max(hi(S.vx[a]), max(hi(S.vy[a]), hi(S.vz[a]))));
     mg = max(mg, hi(S.gm[a]));
+    if (hi(S.gm[a])) lg = min(lg, hi(S.gm[a]));
   }
   GroupScale g;
   g.ea = (int)(__reduce_max_sync(FULL, mx) >> 20) - 1023;
@@ -38,11 +45,13 @@ __device__ GroupScale group_scale(const GView &S, const GroupCtx &C, int lane) {
   if (g.eb < -900) g.eb = ((((__double2hiint(C.mu) >> 20) & 0x7FF) - 1023) - g.ea) / 2;
   bool ok = abs(g.ea) < 400 && abs(g.eb) < 400;
   const int et = -g.ea - 2 * g.eb, eg = (int)(__reduce_max_sync(FULL, mg) >> 20) - 1023 + et;
+  const int el = (int)(__reduce_min_sync(FULL, lg) >> 20) - 1023 + et;        // (large where no body has mass)
+  const int eh = top(C.dp->hk[C.max_depth]) + g.eb - g.ea;
   const float h = fabsf(f32_trunc(scale2(C.dp->hk[1], g.eb - g.ea))), mh = fabsf(f32_trunc(scale2(C.mu, et))) * h * h;
-  ok = ok && h > 1e-18f && h < 1e12f && mh > 1e-28f && mh < 1e12f && eg < 38;
+  ok = ok && h < 1e12f && mh > 1e-28f && mh < 1e12f && eg < 38 && eh >= -70 && el + eh - 1 >= -100;
   for (int q = lane; q < C.pcnt; q += 32) {
-    const float r = f32_trunc(scale2(S.R0[q], -g.ea));
-    ok = ok && r > 1e-12f && r < 1e6f;
+    const int er = top(S.R0[q] * C.dp->ck[C.max_depth + 1]) - g.ea;
+    ok = ok && 3 * -er + max(eg, 0) <= 124 && f32_trunc(scale2(S.R0[q], -g.ea)) < 1e6f;
   }
   g.fits = __all_sync(FULL, ok) != 0;
   return g;

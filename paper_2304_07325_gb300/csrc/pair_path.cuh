@@ -641,12 +641,15 @@ __device__ __forceinline__ int pair_run(const Dev &D, const GroupCtx &C, int lan
         const float need = fM * (speed + fM * (kmax + 4.0f * fabsf(u) * Rp)) * 1.0001f;
         return r.h * 0.9999f > fmaxf(Rj, rcut) + need && r.h * 1.0001f + need < Rp;
       };
-      const bool run = far && substeps + M < max_sub && __all_sync(FULL, clear(hdv, uh));
+      // A run's kick takes G m h^2 / 2 as one number: below 2^-100 its low part is lost (pairs closer than about
+      // 2^-27 of their distance from the sun), and the sub-steps are taken one by one, kick and h apart.
+      const df gh = ld(odd ? T->hb[j] : T->ha[j]);
+      const bool whole = fabsf(gh.h) > 7.8886091e-31f || gg.h == 0.0f;
+      const bool run = far && substeps + M < max_sub && __all_sync(FULL, whole && clear(hdv, uh));
       int end = run ? M : cj + 1;
       substeps += end - 1 - cj;                            // (this one is counted)
       if (order2 && !fresh) sun();
       const bool wide = so >= 1e-8f, beyond = so > 2.0e-6f;
-      const df gh = ld(odd ? T->hb[j] : T->ha[j]);           // G m h^2 / 2
       Run S;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
