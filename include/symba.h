@@ -229,8 +229,10 @@ void symba_pool_free(symba_pool *pool);
 /* groups touch disjoint bodies -- only the time.                                              */
 /* ---------------------------------------------------------------------------------------- */
 typedef struct {
-  int kick_blocks_per_sm;   /* persistent kick CTAs (4 warps each) per multiprocessor, >= 1 */
-  int kick_tiles_per_item;  /* tiles a warp takes per grab from the tile queue, 1..64 */
+  int kick_blocks_per_sm;   /* persistent kick CTAs per multiprocessor, >= 1 (FP64 systems: 16 warps each, up
+                               to 4, of which those beyond the resident ones find the queue empty; mixed:
+                               4 warps each, up to the kernel's occupancy limit) */
+  int kick_tiles_per_item;  /* macro-tiles a CTA takes per grab from the queue, 1..64 */
   int rec_blocks_per_sm;    /* recursion CTAs (4 warps, one per SM quadrant) per SM, 1 or 2 */
   int group_order;          /* 0: groups in label order; 1: longest estimated chain first
                                (M^k for the deepest shell k the pair's straight-line closest
@@ -253,12 +255,12 @@ typedef struct {
 /* Current schedule of a pool (host struct). */
 int symba_pool_get_schedule(symba_pool *pool, symba_schedule *s);
 
-/* Sets a schedule; SYMBA_E_INVAL for fields outside their ranges (kick_blocks_per_sm above the
- * kernel's occupancy limit included).  Takes effect at the next step. */
+/* Sets a schedule; SYMBA_E_INVAL for fields outside their ranges (kick_blocks_per_sm above its
+ * limit included).  Takes effect at the next step. */
 int symba_pool_set_schedule(symba_pool *pool, const symba_schedule *s);
 
 /* Times candidate schedules on the pool's current systems and keeps the fastest; synchronises.
- * Kick: every kick_blocks_per_sm up to the occupancy limit x kick_tiles_per_item in
+ * Kick: every kick_blocks_per_sm up to the number of resident CTAs x kick_tiles_per_item in
  * {1, 2, 4, 8, 16}, each timed over reps (>= 1) launches of the second kick, which writes only
  * per-tile scratch that every step overwrites.  Recursion: rec_blocks_per_sm in {1, 2} x
  * group_order in {0, 1}, each timed on the same trial step, run from a device copy of the

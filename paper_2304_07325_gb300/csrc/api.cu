@@ -780,7 +780,7 @@ int pool_autotune(symba_pool *P, int reps, symba_tune_result *out) {
   if (rc == SYMBA_OK) {
     r.kick_ms_before = time_kick(before.kick_blocks_per_sm, before.kick_tiles_per_item);
     r.kick_ms = r.kick_ms_before;
-    const int kmax = trap_blocks_per_sm(P->precision);
+    const int kmax = trap_blocks_default(P->precision);     // more CTAs than are resident find the queue empty
     for (int kb = 1; kb <= kmax && rc == SYMBA_OK; ++kb) {
       for (int seg : {1, 2, 4, 8, 16}) {
         const double ms = time_kick(kb, seg);
