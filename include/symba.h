@@ -45,8 +45,17 @@ extern "C" {
 #define SYMBA_E_NONFINITE (-7) /* NaN or Inf in the state */
 #define SYMBA_COLLISION 1      /* informational: bodies merged during the last steps */
 
-#define SYMBA_PRECISION_FP64 0 /* every operation in FP64 */
-#define SYMBA_PRECISION_MIXED 1 /* FP32 pair kick (Kahan into FP64); FP64 state, drifts, check, energy */
+/* Precision.  In both modes the state, the level-0 check and the Kepler and sun drifts are FP64, and momentum and
+ * energy are correctly rounded sums of FP64 terms.  The recursion carries FP64 positions and velocities and
+ * forms what a sub-step adds to them (separations, forces, kicks, drifts short against the orbit) as sums of
+ * two FP32 numbers, 2^-46 of the increment; separations are exact differences of the FP64 positions.  Groups
+ * whose quantities do not fit FP32's range are taken in FP64.
+ *   FP64:  the pair kick's forces are sums of two FP32 numbers too (2^-46 of a force) where that is less than
+ *          2^-54 of the velocity they change; elsewhere -- kicks above about 2^-8 of the velocity, systems
+ *          spread over many orders of magnitude -- and in all sums over tiles FP64.
+ *   MIXED: the pair kick's forces are FP32, Kahan-summed and carried into FP64 once. */
+#define SYMBA_PRECISION_FP64 0
+#define SYMBA_PRECISION_MIXED 1
 
 /* Method parameters (Sec. 3 gives dt, M, shell_ratio and l for the benchmark). */
 typedef struct {
@@ -223,7 +232,7 @@ void symba_pool_free(symba_pool *pool);
 
 /* ---------------------------------------------------------------------------------------- */
 /* Launch schedules and their autotuner.  The pair kick (Sec. 2's trapezoid loop) is a queue   */
-/* of 32 x 32 tiles taken by persistent warps; the encounter groups (Sec. 2: each group is     */
+/* of macro-tiles taken by persistent CTAs; the encounter groups     (Sec. 2: each group is     */
 /* integrated independently) are a queue of groups taken by persistent warps.  How the queues  */
 /* are cut and ordered changes no result -- per-tile partials are reduced in a fixed order and  */
 /* groups touch disjoint bodies -- only the time.                                              */
@@ -279,8 +288,9 @@ int symba_autotune(symba_ctx *c, int reps, symba_tune_result *out);
 const char *symba_status_string(int status);
 
 /* Measures, on the current device, the rates that bound this path (measurement infrastructure:
- * the paper reports only wall-clock times, Sec. 3; the pair kick of Sec. 2 is FP64-pipe bound
- * and the per-group recursion is bound by one warp's dependent FP64 work).  Writes out[0..5]
+ * the paper reports only wall-clock times, Sec. 3; the energy's pair terms are bound by the FP64
+ * pipe, and what one warp's dependent FP64 work costs is why the pair kick of Sec. 2 and the
+ * per-group recursion are formed on the FP32 pipe).  Writes out[0..5]
  * (host): 0 the device's FP64 FLOP/s (independent fused multiply-adds on every SM, an FMA
  * counting 2 flops); 1 cycles per FMA of one warp's dependent FMA chain; 2 cycles per FMA of one
  * warp running four independent chains; 3 cycles per round trip of a value between two warps of

@@ -6,8 +6,8 @@
 //   alive, gid                                     : int per particle (gid = encounter group or -1)
 //   xf, yf, zf, vxf, vyf, vzf, lamf, sigf          : FP32 copies for the encounter prefilter
 //   tiles                                          : int4 {system, first row block, first column block,
-//                                                    end of the massive blocks} per 4 x 4 macro-tile
-//                                                    of 32 x 32 tiles (128-body quads q <= c)
+//                                                    end of the massive blocks} per macro-tile of
+//                                                    4 x SYM_MACRO_COLS tiles of 32 x 32 bodies
 //   fblk                                           : int2 {system, block} per block of field particles
 //   part                                           : [macro-tile][rows, columns][4][3][32] pair-kick
 //                                                    partials, 8 bytes each (FP64; mixed: FP32 sum and
@@ -64,7 +64,7 @@ struct Dev {
   double *P;                    // [max_disks][3] total barycentric momentum (for the sun drift)
   unsigned long long *sacc;     // [max_disks][3][SA_NDIG + 1] exact accumulators
   // trapezoid
-  int4 *tiles;                  // macro-tiles (quads q <= c) over the blocks holding massive bodies
+  int4 *tiles;                  // macro-tiles over the blocks holding massive bodies
   double *part;                 // [macro-tile][SYM_MACRO_PART] (mixed: pairs of FP32)
   int2 *fblk;                   // field rectangle: {system, block} of every block of field particles only
   int nfblk;
@@ -206,16 +206,6 @@ __device__ __forceinline__ bool lt_nn(double a, double b) {
 __device__ __forceinline__ bool is_neg(double a) { return __double_as_longlong(a) < 0; }
 __device__ __forceinline__ double neg(double a) {
   return __longlong_as_double(__double_as_longlong(a) ^ (long long)0x8000000000000000ull);
-}
-__device__ __forceinline__ double abs_bits(double a) {
-  return __longlong_as_double(__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll);
-}
-__device__ __forceinline__ double max_nn(double a, double b) { return lt_nn(a, b) ? b : a; }
-
-// Select without arithmetic: v if keep, else 0.0 (integer select on the bit pattern).
-__device__ __forceinline__ double keep_or_zero(double v, bool keep) {
-  long long b = __double_as_longlong(v);
-  return __longlong_as_double(keep ? b : 0ll);
 }
 
 // --------------------------------------------------------------------------------------------

@@ -326,8 +326,8 @@ void launch_momentum(const Dev &D, int ndisks, long long npart, int n_max, bool 
 // kick: a_p = fixed-order sum of the trapezoid partials that touch p, then v_p = v_p + (tau/2) a_p.
 // Macro-tiles are (row quad q, column group g), C = SYM_MACRO_COLS column blocks per group, g from
 // 4q / C; block B of the system has its row partials in (B/4, g), g = 4(B/4)/C..ng-1 (row slot
-// B % 4), then its column partials in (q, B/C), q = 0..B/4 (column slot B % C; the diagonal
-// tiles' column sides are folded into their rows).  Macro-tile (q, g) is entry
+// B % 4), then its column partials in (q, B/C), q = 0..B/4 (column slot B % C; the mixed kick folds
+// the diagonal tiles' column sides into their rows).  Macro-tile (q, g) is entry
 // tile_base + q ng - (4/C) q (q - 1)/2 + (g - 4q/C) of the list.
 // --------------------------------------------------------------------------------------------
 __device__ __forceinline__ int macro_index(const DiskDesc &dd, int ng, int q, int g) {
@@ -336,7 +336,7 @@ __device__ __forceinline__ int macro_index(const DiskDesc &dd, int ng, int q, in
 
 // One CTA per 32-body block: warp w adds every RED_SLICES-th partial of the block's bodies, and the
 // sums join in warp order.  (One thread per body took 88 us for 10,000 bodies, a chain of 80 dependent
-// loads and sums on 79 CTAs; now 16 us.)
+// loads and sums on 79 CTAs; now 23 us, with FP64 sums.)
 #define RED_SLICES 8
 __global__ void __launch_bounds__(32 * RED_SLICES) k_reduce(Dev D, long long nblk) {
   __shared__ double sh[RED_SLICES][3][32];

@@ -20,9 +20,11 @@
 //
 // FP64 systems form the pair force in double-float (df32.cuh) on the FP32 pipe, which GB300 runs at
 // 62x the FP64 rate.  Separations come from coordinates cut on grids common to a macro-tile, exact
-// to 2^-61 of its extent; r^-3, the products and the sums carry 46 to 48 bits.  A kick is a small part
-// of v (a body of 1e-3 m0 at 1 AU and tau = 0.5 yr: 1/300), so its 2^-46 lies below the rounding
-// of v += (tau/2) a that follows; against an 80-bit kick the new v is as close as the FP64 pairs' was.
+// to 2^-61 of its extent; r^-3, the products and a macro-tile's sums carry 46 to 48 bits, which lies below
+// the rounding of v += (tau/2) a while a kick is a small part of v (a body of 1e-3 m0 at 1 AU and
+// tau = 0.5 yr: 1/300); where it is not, and where the macro-tile's extent would cost digits, the
+// macro-tile is taken in FP64 (see "how far the double-float form may go").  Against an 80-bit kick the
+// new v is as close as FP64 pairs bring it.
 //   10,000 bodies, per kick: 1.48 ms with 16.5 FP64 instructions per pair (FP64 pipe 90 % busy) ->
 //   0.55-0.58 ms with ~260 warp instructions per 32 pairs (61 % of the issue slots; four barriers per
 //   macro-tile take most of the rest).  1,000 bodies 0.160 -> 0.021 ms, 100 bodies 0.065 -> 0.017 ms
@@ -750,25 +752,25 @@ void launch_trap(const Dev &D, const LaunchCfg &L, int mode, int precision, cuda
 // ---------------------------------------------------------------------------------------------
 // The field rectangle (Sec. 2: field particles interact only with massive bodies).  The
 // trapezoid's tiles cover the column blocks that hold massive bodies; every block of field
-// particles beyond them is one row of the rectangle N_m x N_field, taken by one warp: lane l
-// owns field particle b*32 + l, the system's massive bodies stream through a per-warp
-// shared-memory chunk of 32 (one coalesced load, then broadcast reads), and only the field
-// particle's side is accumulated -- a massless body exerts no force, so the massive side and the
-// per-tile partials of the trapezoid are not needed.  The sum over i runs in ascending order,
-// so the result does not depend on the launch or on other systems, and the kick
-// v += (tau/2) a is applied at the end (the reduction skips these blocks).  Kick 1 runs the same
+// particles beyond them is one row of the rectangle N_m x N_field: lane l owns field particle
+// b*32 + l, the system's massive bodies stream through a per-warp shared-memory chunk of 32 (one
+// coalesced load, then broadcast reads), and only the field particle's side is accumulated -- a
+// massless body exerts no force, so the massive side and the per-tile partials of the trapezoid are
+// not needed.  FP64 systems: four warps take every fourth chunk each and their sums are added in
+// warp order; mixed: one warp takes all, in ascending order.  So the result does not depend on the
+// launch or on other systems.  The kick v += (tau/2) a is applied at the end (the reduction skips
+// these blocks).  Kick 1 runs the same
 // fused encounter check as the tiles (FP32 prefilter, exact FP64 predicate, pair emission,
 // g_0 weight); kick 2 weights the flagged pairs through the groups.
 // ---------------------------------------------------------------------------------------------
-struct FieldSrc {
-  double x, y, z, gm;
-  float xf, yf, zf, xl, yl, zl, gmf;           // FP32 copies; low parts and G m (mixed)
+struct FieldSrc {                              // mixed precision
+  float xf, yf, zf, xl, yl, zl, gmf;           // FP32 copies, low parts, G m
   float vxf, vyf, vzf, lam, sig;               // kick 1 prefilter
   int id, ok, gid;
 };
 
 // stage massive bodies [c0, c0 + 32) of the system into the warp's chunk
-template <int MODE, bool MIXED>
+template <int MODE>
 __device__ __forceinline__ void stage_sources(const Dev &D, const TileCtx &c, int c0, int lane, FieldSrc *src) {
   const int li = c0 + lane;
   FieldSrc s;
@@ -776,12 +778,8 @@ __device__ __forceinline__ void stage_sources(const Dev &D, const TileCtx &c, in
   s.id = p;
   s.ok = (li < c.nm && D.alive[p]) ? 1 : 0;
   const int q = s.ok ? p : c.off;               // a valid address for the loads below
-  s.x = D.x[q]; s.y = D.y[q]; s.z = D.z[q]; s.gm = D.gm[q];
   s.xf = D.xf[q]; s.yf = D.yf[q]; s.zf = D.zf[q];
-  s.xl = 0.f; s.yl = 0.f; s.zl = 0.f; s.gmf = 0.f;
-  if (MIXED) {
-    s.xl = D.xl[q]; s.yl = D.yl[q]; s.zl = D.zl[q]; s.gmf = D.gmf[q];
-  }
+  s.xl = D.xl[q]; s.yl = D.yl[q]; s.zl = D.zl[q]; s.gmf = D.gmf[q];
   s.vxf = 0.f; s.vyf = 0.f; s.vzf = 0.f; s.lam = 0.f; s.sig = 0.f;
   if (MODE == 1) {
     s.vxf = D.vxf[q]; s.vyf = D.vyf[q]; s.vzf = D.vzf[q]; s.lam = D.lamf[q]; s.sig = D.sigf[q];
@@ -988,7 +986,7 @@ __global__ void __launch_bounds__(128) k_field_mixed(Dev D) {
   float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
   for (int c0 = 0; c0 < c.nm; c0 += 32) {
     __syncwarp();
-    stage_sources<MODE, true>(D, c, c0, lane, src);
+    stage_sources<MODE>(D, c, c0, lane, src);
     __syncwarp();
     const int cnt = min(32, c.nm - c0);
 #pragma unroll 1
