@@ -36,13 +36,18 @@ FLOPS_PER_PAIR_CHECK = 18
 INSTR_PER_PAIR_SUBSTEP = 335.9
 INSTR_PER_GENERAL_SUBSTEP = 4942.7
 # and of the FP64 pair kick per pair: mean of kick 1 and kick 2 (profiles/k_trap_df_disk_N10000.md)
-INSTR_PER_PAIR_KICK = (428516403 + 388191833) / 2 / 49995000
+INSTR_PER_PAIR_KICK = (450647336 + 409993064) / 2 / 49995000
+# what dtype stands for
+ARITHMETIC = ["FP64 state, drifts, checks and sums; pair forces as sums of two FP32 numbers where that is below the "
+              "rounding of the velocity, FP64 elsewhere; recursion increments as sums of two FP32 numbers",
+              "FP64 state, drifts, checks and sums; FP32 pair kick (Kahan into FP64); recursion increments as sums of "
+              "two FP32 numbers"]
 # The recursion of the bound-pair group the profiles use (bodies of the N = 10,000 disk, seed 1002)
 BOUND_PAIR_GROUP = [1244, 3406, 4643, 5122, 9870]
 # DRAM read + write per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum, N = 10,000, FP64)
 # of the current kernels; None until a capture of the current kernel is on record
 RECURSION_TRAFFIC_BYTES = 1388288 + 6144       # first step of the disk (profiles/k_recursion_disk_N10000.md)
-KICK_TRAFFIC_BYTES = ((1154560 + 0) + (730112 + 0)) / 2          # kick 1, kick 2 (profiles/k_trap_df_disk_N10000.md)
+KICK_TRAFFIC_BYTES = ((1169408 + 1024) + (987648 + 0)) / 2          # kick 1, kick 2 (profiles/k_trap_df_disk_N10000.md)
 # Step size at which the batched and served forms and the one-at-a-time form all keep the energy
 # error of every merger-free disk below 1e-10 (measured on the 64 batched disks: 5.7e-11 after 20
 # steps at 0.125 yr, 1.1e-10 at 0.2, 5.2e-10 at 0.5)
@@ -688,7 +693,8 @@ def run_ours(args):
         line = {"metric": "pair-interactions/s", "value": value, "unit": "pair-interactions/s",
                 "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
                 "ms_per_step": 1e3 * t_max / args.steps, "higher_is_better": True, "scaling": "weak",
-                "vs_baseline": None, "dtype": "f64" if prec == 0 else "f32-pair/f64-state", "data": "synthetic",
+                "vs_baseline": None, "dtype": "f64" if prec == 0 else "f32-pair/f64-state",
+                "arithmetic": ARITHMETIC[prec], "data": "synthetic",
                 "config": {"workload": workload_name(args),
                            "seeds": f"{args.seed} + 1000 * rank (replicas)" if world > 1 else str(args.seed),
                            "n": args.n, "pairs_per_kick": P, "l2": "flushed between steps (256 MB write)"

@@ -26,9 +26,9 @@
 // macro-tile is taken in FP64 (see "how far the double-float form may go").  Against an 80-bit kick the
 // new v is as close as FP64 pairs bring it.
 //   10,000 bodies, per kick: 1.48 ms with 16.5 FP64 instructions per pair (FP64 pipe 90 % busy) ->
-//   0.55-0.58 ms with ~260 warp instructions per 32 pairs (61 % of the issue slots; four barriers per
-//   macro-tile take most of the rest).  1,000 bodies 0.160 -> 0.021 ms, 100 bodies 0.065 -> 0.017 ms
-//   (see k_trap_df and launch_trap for the small systems).
+//   0.50-0.57 ms with ~275 warp instructions per 32 pairs (60 % of the issue slots; four barriers per
+//   macro-tile take most of the rest); 3.1 ms when every macro-tile is taken in FP64.  1,000 bodies
+//   0.160 -> 0.019 ms, 100 bodies 0.065 -> 0.018 ms (see k_trap_df and launch_trap for the small systems).
 //
 // Kick 1 also runs the close-encounter check (Sec. 2) of every pair: a conservative FP32
 // prefilter (|d| - tau |dv| against R_0 with rounding margins) and, for the rare pairs that pass,
