@@ -182,3 +182,34 @@ def test_flagged_pairs_beside_a_far_body(orc, sy, nf):
         rel = (np.linalg.norm(a - b, axis=1) / np.linalg.norm(b, axis=1))[live]
         spread = (np.linalg.norm(t - b, axis=1) / np.linalg.norm(b, axis=1))[live]
         assert np.all(rel <= np.maximum(1e-13, 100.0 * spread)), float((rel / np.maximum(1e-13, 100.0 * spread)).max())
+
+
+def test_neighbours_and_schedules_change_no_bit(sy):
+    """Systems with macro-tiles taken in FP64, alone, in one pool with an ordinary one, and with several
+    macro-tiles per grab."""
+    ds = []
+    for n, nf, far in ((300, 80, True), (500, 0, False), (700, 200, True)):
+        x, v, m = heavy_disk(n, 50 + n, nf)
+        if far:
+            for k in range(20, n + nf, 150):
+                x[k] *= 1e9
+                v[k] /= math.sqrt(1e9)
+        ds.append((x, v, m, n))
+    params = sy.default_params(hill_scale=0.0, dt=0.05)
+    alone = []
+    for x, v, m, n in ds:
+        s = sy.System(x, v, m, np.zeros(len(m)), n_massive=n, params=params)
+        s.step(3)
+        assert s.sync() >= 0
+        alone.append(s.get_state())
+        s.close()
+    tiles = sum(((len(m) + 31) // 32) ** 2 for _, _, m, _ in ds)
+    for per_item in (1, 16):
+        pool = sy.Pool(3, sum(len(m) for _, _, m, _ in ds), tiles)
+        slots = [pool.admit(x, v, m, np.zeros(len(m)), n_massive=n, params=params) for x, v, m, n in ds]
+        pool.schedule = dict(pool.schedule, kick_tiles_per_item=per_item)
+        pool.step(3)
+        assert pool.sync() >= 0
+        for k, want in zip(slots, alone):
+            assert all(np.array_equal(a, b) for a, b in zip(pool.get_state(k), want))
+        pool.close()
